@@ -87,7 +87,8 @@ def draw(rng):
         return {"op": op, "prec": rng.choice(["f16", "f16", "f32"]), "nrhs": rng.randint(2, 16),
                 "dims": ",".join(_dims(rng, 512, mid // 2) for _ in range(rng.randint(1, 3)))}
     if op == "multi":
-        return {"op": op, "prec": rng.choice(["f16", "f32"]), "nrhs": rng.randint(2, 20), "dims": _dims(rng, 256, mid // 2)}
+        prec = rng.choice(["f16", "f32"])
+        return {"op": op, "prec": prec, "nrhs": rng.randint(2, 20), "dims": _dims(rng, 256, mid // 2)}
     if op == "ptc":
         return {"op": op, "dims": _dims(rng, 256, mid)}
     if op == "ptc_train":
@@ -177,6 +178,17 @@ def _import(lat, prec, spinors, parity=dirac.PARITY_FULL):
     return x
 
 
+def _numbers(lat, f, prec):
+    """The numbers of a field, as the library lays them out."""
+    if prec == dirac.F64:
+        return f.view(torch.float64)
+    if prec == dirac.F32:
+        return f.view(torch.float32)
+    vh, w = lat.volume // 2, 2 * lat.nr  # 16-bit values of a half-field, then its per-site norms
+    f = f.view(-1, (w + 4) * vh)
+    return [f[:, :w * vh].view(torch.float16), f[:, w * vh:].view(torch.float32)]
+
+
 def prepare(case, seed):
     op = case["op"]
     solve = op in ("cg", "gcr_dd", "bicgstab_many")
@@ -184,7 +196,7 @@ def prepare(case, seed):
     mask = {"cg": 1, "gcr_dd": 5, "bicgstab_many": 5}.get(op, 1 << prec)
     parity = dirac.PARITY_EVEN if op in ("asqtad", "eo") else dirac.PARITY_FULL
     st = {"op": op, "prec": prec, "parity": parity, "nrhs": case.get("nrhs", 1), "dagger": case.get("dagger", False),
-          "lats": [], "ins": [], "outs": []}
+          "lats": [], "ins": [], "outs": [], "numbers": []}
     for l, (dims, fields) in enumerate(zip(_lattices(case), _natural(case, seed))):
         if op == "asqtad":
             lat = dirac.Lattice(dims, dirac.ASQTAD, mass=MASS, prec_mask=mask)
@@ -197,6 +209,7 @@ def prepare(case, seed):
         st["lats"].append(lat)
         st["ins"].append(_import(lat, prec, fields[-1], parity))
         st["outs"].append(torch.zeros_like(st["ins"][-1]))
+        st["numbers"].append(_numbers(lat, st["outs"][-1], prec))
     if op == "batch":
         st["plan"] = dirac.Batch(st["lats"], st["outs"], st["ins"], [st["nrhs"]] * len(st["lats"]), prec)
     if op in ("ptc", "ptc_train"):
@@ -210,19 +223,6 @@ def prepare(case, seed):
 
 
 # -------------------------------------------------------------------------------- run
-def _numbers(st, l):
-    """The numbers of an output field, as the library lays them out."""
-    f, prec = st["outs"][l], st["prec"]
-    if prec == dirac.F64:
-        return f.view(torch.float64)
-    if prec == dirac.F32:
-        return f.view(torch.float32)
-    lat = st["lats"][l]
-    vh, w = lat.volume // 2, 2 * lat.nr  # 16-bit values of a half-field, then its per-site norms
-    f = f.view(-1, (w + 4) * vh)
-    return [f[:, :w * vh].view(torch.float16), f[:, w * vh:].view(torch.float32)]
-
-
 def run(st):
     op, lat, x, y, prec = st["op"], st["lats"][0], st["ins"][0], st["outs"][0], st["prec"]
     if op == "m":
@@ -252,7 +252,7 @@ def run(st):
     else:
         dirac.solve_many(st["lats"], st["outs"], st["ins"], [st["nrhs"]] * len(st["lats"]), tol=TOL, delta=0.1,
                          prec_sloppy=dirac.F16)
-    return [_numbers(st, l) for l in range(len(st["lats"]))]
+    return st["numbers"]
 
 
 # ------------------------------------------------------------------------------- work
