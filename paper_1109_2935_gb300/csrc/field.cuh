@@ -8,6 +8,7 @@
 #pragma once
 #include <cuda_fp16.h>
 #include <cstdint>
+#include <type_traits>
 
 namespace dirac {
 
@@ -65,12 +66,24 @@ template <typename T> __device__ __forceinline__ void cmacc(C<T>& a, C<T> b, C<T
 
 template <typename T> struct Link { C<T> m[3][3]; };
 
+// The first products of a row: u h (CONJ: conj(u) h). In FP64 every step is a product or a
+// fused multiply-add as written (the compiler has no choice of contraction), so that
+// U^dagger h equals W h for W = U^dagger bit for bit (wilson_split.cuh needs it).
+template <bool CONJ, typename T> __device__ __forceinline__ C<T> cmul0(C<T> u, C<T> h) {
+  if constexpr (sizeof(T) == 8 && std::is_floating_point<T>::value) {
+    const T ui = CONJ ? -u.i : u.i;
+    return C<T>{fma(u.r, h.r, -(ui * h.i)), fma(ui, h.r, u.r * h.i)};
+  } else {
+    return (CONJ ? conj(u) : u) * h;
+  }
+}
+
 // v = U h (3-vector)
 template <typename T>
 __device__ __forceinline__ void su3_mv(const Link<T>& U, const C<T> h[3], C<T> v[3]) {
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    v[a] = U.m[a][0] * h[0];
+    v[a] = cmul0<false>(U.m[a][0], h[0]);
     cmac(v[a], U.m[a][1], h[1]);
     cmac(v[a], U.m[a][2], h[2]);
   }
@@ -80,7 +93,7 @@ template <typename T>
 __device__ __forceinline__ void su3_mv_dag(const Link<T>& U, const C<T> h[3], C<T> v[3]) {
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    v[a] = conj(U.m[0][a]) * h[0];
+    v[a] = cmul0<true>(U.m[0][a], h[0]);
     cmacc(v[a], U.m[1][a], h[1]);
     cmacc(v[a], U.m[2][a], h[2]);
   }

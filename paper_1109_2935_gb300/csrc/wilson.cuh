@@ -290,6 +290,24 @@ template <> struct WilsonShape<P32> { static constexpr int threads = 64, minb = 
 template <> struct WilsonShape<P64> { static constexpr int threads = 128, minb = 1; };
 template <> struct WilsonShape<P64DS> { static constexpr int threads = 128, minb = 2; };
 
+// Output site idx of the full operator. The two parities alternate every
+// WILSON_INTERLEAVE threads (a warp: the parity stays warp-uniform): the forward link
+// U_mu(x) read by site x is read again as a backward link by the neighbour x + mu of the
+// other parity close in time, so it comes from cache instead of a second DRAM pass over
+// all links.
+__device__ __forceinline__ void full_site(int idx, int Vh, int& par, int& cb) {
+  constexpr int IL = WILSON_INTERLEAVE;
+  const int grp = idx / (2 * IL), k = idx - grp * 2 * IL;
+  if ((grp + 1) * IL <= Vh) {
+    par = k >= IL;
+    cb = grp * IL + k - par * IL;
+  } else {  // last, incomplete pair of groups (Vh not a multiple of IL)
+    const int half = Vh - grp * IL;
+    par = k >= half;
+    cb = grp * IL + k - par * half;
+  }
+}
+
 // One output site of the stencil: thread index idx over the Vh (hop mode) or 2 Vh
 // (full operator) output sites. Shared by the single-RHS, multi-RHS and batched kernels.
 template <int PREC, int R, bool FULLM>
@@ -299,21 +317,8 @@ __device__ __forceinline__ void wilson_site(const WilsonArg& a, int idx) {
   const int Vh = g.Vh;
   int par, cb;
   if (FULLM) {
-    // The two parities alternate every WILSON_INTERLEAVE threads (a warp: the parity
-    // stays warp-uniform): the forward link U_mu(x) read by site x is read again as a
-    // backward link by the neighbour x + mu of the other parity close in time, so it
-    // comes from cache instead of a second DRAM pass over all links.
     if (idx >= 2 * Vh) return;
-    constexpr int IL = WILSON_INTERLEAVE;
-    const int grp = idx / (2 * IL), k = idx - grp * 2 * IL;
-    if ((grp + 1) * IL <= Vh) {
-      par = k >= IL;
-      cb = grp * IL + k - par * IL;
-    } else {  // last, incomplete pair of groups (Vh not a multiple of IL)
-      const int half = Vh - grp * IL;
-      par = k >= half;
-      cb = grp * IL + k - par * half;
-    }
+    full_site(idx, Vh, par, cb);
   } else {
     if (idx >= Vh) return;
     par = a.out_parity;
