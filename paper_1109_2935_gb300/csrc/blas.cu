@@ -53,7 +53,7 @@ const char* blas_error(Blas* b) { return b ? b->err.c_str() : "no blas context";
 
 // ---------------------------------------------------------------- site access
 template <int NR, typename T>
-__device__ __forceinline__ void site_load(const FieldRef& f, int s, T v[NR]) {
+__device__ __forceinline__ void any_load(const FieldRef& f, int s, T v[NR]) {
   int q = s >= f.Vh ? 1 : 0;
   int cb = s - q * f.Vh;
   const char* b = f.p + q * f.hb;
@@ -76,7 +76,7 @@ __device__ __forceinline__ void site_load(const FieldRef& f, int s, T v[NR]) {
 }
 
 template <int NR, typename T>
-__device__ __forceinline__ void site_store(const FieldRef& f, int s, const T v[NR]) {
+__device__ __forceinline__ void any_store(const FieldRef& f, int s, const T v[NR]) {
   int q = s >= f.Vh ? 1 : 0;
   int cb = s - q * f.Vh;
   char* b = f.p + q * f.hb;
@@ -94,11 +94,33 @@ __device__ __forceinline__ void site_store(const FieldRef& f, int s, const T v[N
   }
 }
 
+// The NR reals of "site" s: a lattice site, or with NR = 2 (operations on FP64 fields only)
+// 16-byte chunk s of the half-fields one after the other.
+template <int NR, typename T>
+__device__ __forceinline__ void site_load(const FieldRef& f, int s, T v[NR]) {
+  if constexpr (NR == 2) {
+    const double2 t = reinterpret_cast<const double2*>(f.p)[s];
+    v[0] = t.x;
+    v[1] = t.y;
+  } else {
+    any_load<NR>(f, s, v);
+  }
+}
+template <int NR, typename T>
+__device__ __forceinline__ void site_store(const FieldRef& f, int s, const T v[NR]) {
+  if constexpr (NR == 2) reinterpret_cast<double2*>(f.p)[s] = make_double2(v[0], v[1]);
+  else any_store<NR>(f, s, v);
+}
+
 // Stores v like site_store and leaves in v the values as stored, so that a reduction
 // over the result needs no reload: for FP16 the binary16 values times the per-site
 // norm, computed exactly as a load decodes them; FP32 / FP64 storage leaves v as it is.
 template <int NR, typename T>
 __device__ __forceinline__ void site_store_q(const FieldRef& f, int s, T v[NR]) {
+  if constexpr (NR == 2) {
+    site_store<NR>(f, s, v);
+    return;
+  }
   if (f.prec != P16) {
     site_store<NR>(f, s, v);
     return;
@@ -619,27 +641,32 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<Op>::value) blas_map_kerne
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) op(i, nullptr);
 }
 
-__device__ __forceinline__ double warp_sum(double v) {
+// Sums of three values over a block, left in sum[0..2] of shared memory (valid after the
+// call). Warp k < 3 adds value k: 7 + 5 dependent FP64 additions. FP64 instructions issue at
+// one per 64 cycles and scheduler on this part whatever the active lanes, so shuffles in
+// all 8 warps followed by a serial pass over their results (39 per warp and 24 in thread 0)
+// took 1.7 us of every block; this takes 0.4.
+struct RedShared {
+  double v[3][kThreads];
+  double sum[3];
+  bool last;
+};
+__device__ __forceinline__ void block_sum3(const double acc[3], RedShared& sh) {
+  const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Block sum of three values; the result is valid in thread 0.
-__device__ __forceinline__ void block_sum3(double acc[3], double (*sh)[3]) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) acc[k] = warp_sum(acc[k]);
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) sh[warp][k] = acc[k];
+  for (int j = 0; j < 3; ++j) sh.v[j][threadIdx.x] = acc[j];
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < 3; ++k) {
-      double s = 0;
-      for (int w = 0; w < kThreads / 32; ++w) s += sh[w][k];
-      acc[k] = s;
-    }
+  if (k < 3) {
+    double t[kThreads / 32];
+#pragma unroll
+    for (int j = 0; j < kThreads / 32; ++j) t[j] = sh.v[k][lane + 32 * j];
+#pragma unroll
+    for (int w = kThreads / 64; w > 0; w >>= 1)
+#pragma unroll
+      for (int j = 0; j < w; ++j) t[j] += t[j + w];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t[0] += __shfl_xor_sync(0xffffffffu, t[0], o);
+    if (lane == 0) sh.sum[k] = t[0];
   }
   __syncthreads();
 }
@@ -647,38 +674,30 @@ __device__ __forceinline__ void block_sum3(double acc[3], double (*sh)[3]) {
 template <class Op>
 __global__ void __launch_bounds__(kThreads, MinBlocks<Op>::value) blas_reduce_kernel(Op op, int n, double* partials,
                                                           unsigned* ticket, double* res) {
-  __shared__ double sh[kThreads / 32][3];
-  __shared__ bool last;
+  __shared__ RedShared sh;
   double acc[3] = {0, 0, 0};
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) op(i, acc);
   block_sum3(acc, sh);
   if (threadIdx.x == 0) {
-    for (int k = 0; k < 3; ++k) partials[3 * blockIdx.x + k] = acc[k];
+    for (int k = 0; k < 3; ++k) partials[3 * blockIdx.x + k] = sh.sum[k];
     __threadfence();
-    unsigned t = atomicAdd(ticket, 1u);
-    last = (t == gridDim.x - 1);
+    sh.last = atomicAdd(ticket, 1u) == gridDim.x - 1;
   }
   __syncthreads();
-  if (!last) return;
+  if (!sh.last) return;
   __threadfence();
+  // the last block: thread t takes the partial sums t, t + kThreads, ... of every value
   double s[3] = {0, 0, 0};
   for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
 #pragma unroll
     for (int k = 0; k < 3; ++k) s[k] += __ldcg(partials + 3 * b + k);
   block_sum3(s, sh);
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < 3; ++k) res[k] = s[k];
-    *ticket = 0;
-  }
+  if (threadIdx.x < 3) res[threadIdx.x] = sh.sum[threadIdx.x];
+  if (threadIdx.x == 0) *ticket = 0;
 }
 
 // ---------------------------------------------------------------- host dispatch
 static int nsites(const FieldRef& f) { return f.npar * f.Vh; }
-
-static bool any64(std::initializer_list<const FieldRef*> fs) {
-  for (auto f : fs) if (f->prec == P64) return true;
-  return false;
-}
 
 static int check(Blas* b, const char* what) {
   cudaError_t e = cudaGetLastError();
@@ -720,10 +739,35 @@ static int run_reduce(Blas* b, const Op& op, int n, double* out, int nout, cudaS
   return DIRAC_OK;
 }
 
-// Dispatch on (reals per site, arithmetic type).
-#define DISPATCH(nr, dbl, BODY)                               \
+// Storage of an operation's fields: 0 no FP64, 1 FP64 and others (FP64 arithmetic), 2 FP64
+// only: chunk by chunk (NR = 2; a thread per site would issue 12 x the FP64 instructions in
+// a row, each 64 cycles: CG update on 4^4 20.7 us).
+enum : int { NO64 = 0, SOME64 = 1, ALL64 = 2 };
+static int kind(std::initializer_list<const FieldRef*> fs) {
+  bool all = true, some = false;
+  for (auto f : fs) {
+    all = all && f->prec == P64;
+    some = some || f->prec == P64;
+  }
+  const FieldRef& f = **fs.begin();
+  all = all && (int64_t)nsites(f) * (f.nr / 2) < ((int64_t)1 << 30);  // NS is an int
+  return all ? ALL64 : some ? SOME64 : NO64;
+}
+
+// Dispatch on a field's reals per site and its operation's kind: BODY (which returns) sees
+// NS "sites" of NR reals and the arithmetic type T.
+#define DISPATCH(f, KIND, BODY)                               \
   do {                                                        \
-    if ((nr) == 24) {                                         \
+    const int kind_ = (KIND), ns_ = nsites(f);                \
+    if (kind_ == ALL64) {                                     \
+      constexpr int NR = 2;                                   \
+      using T = double;                                       \
+      const int NS = ns_ * ((f).nr / 2);                      \
+      BODY;                                                   \
+    }                                                         \
+    const int NS = ns_;                                       \
+    const bool dbl = kind_ != NO64;                           \
+    if ((f).nr == 24) {                                       \
       constexpr int NR = 24;                                  \
       if (dbl) { using T = double; BODY; } else { using T = float; BODY; } \
     } else {                                                  \
@@ -733,67 +777,67 @@ static int run_reduce(Blas* b, const Op& op, int n, double* out, int nout, cudaS
   } while (0)
 
 int blas_copy(Blas* b, const FieldRef& dst, const FieldRef& src, cudaStream_t st) {
-  DISPATCH(dst.nr, any64({&dst, &src}), return run_map(b, (OpCopy<NR, T>{dst, src}), nsites(dst), st));
+  DISPATCH(dst, kind({&dst, &src}), return run_map(b, (OpCopy<NR, T>{dst, src}), NS, st));
 }
 int blas_zero(Blas* b, const FieldRef& x, cudaStream_t st) {
   if (cudaMemsetAsync(x.p, 0, x.hb * x.npar, st) != cudaSuccess) return check(b, "memset");
   return DIRAC_OK;
 }
 int blas_axpby(Blas* b, Cf a, const FieldRef& x, Cf bb, const FieldRef& y, cudaStream_t st) {
-  DISPATCH(y.nr, any64({&x, &y}), return run_map(b, (OpAxpby<NR, T>{x, y, a, bb}), nsites(y), st));
+  DISPATCH(y, kind({&x, &y}), return run_map(b, (OpAxpby<NR, T>{x, y, a, bb}), NS, st));
 }
 int blas_pupdate(Blas* b, const FieldRef& r, Cf beta, Cf c, const FieldRef& v, const FieldRef& p,
                  cudaStream_t st) {
   if (all_h24({&r, &v, &p})) return run_map(b, (OpPUpdateH{r, v, p, beta, c}), nsites(p), st);
-  DISPATCH(p.nr, any64({&r, &v, &p}), return run_map(b, (OpPUpdate<NR, T>{r, v, p, beta, c}), nsites(p), st));
+  DISPATCH(p, kind({&r, &v, &p}), return run_map(b, (OpPUpdate<NR, T>{r, v, p, beta, c}), NS, st));
 }
 int blas_norm2(Blas* b, const FieldRef& x, double* out, cudaStream_t st, double* dres) {
-  DISPATCH(x.nr, any64({&x}), return run_reduce(b, (OpNorm2<NR, T>{x}), nsites(x), out, 1, st, dres));
+  DISPATCH(x, kind({&x}), return run_reduce(b, (OpNorm2<NR, T>{x}), NS, out, 1, st, dres));
 }
 int blas_cdot(Blas* b, const FieldRef& x, const FieldRef& y, double out[2], cudaStream_t st, double* dres) {
   if (all_h24({&x, &y})) return run_reduce(b, (OpCdotNormH{x, y}), nsites(x), out, 2, st, dres);
-  DISPATCH(x.nr, any64({&x, &y}),
-           return run_reduce(b, (OpCdotNorm<NR, T>{x, y}), nsites(x), out, 2, st, dres));
+  DISPATCH(x, kind({&x, &y}),
+           return run_reduce(b, (OpCdotNorm<NR, T>{x, y}), NS, out, 2, st, dres));
 }
 int blas_cdot_norm(Blas* b, const FieldRef& x, const FieldRef& y, double out[3], cudaStream_t st,
                    double* dres) {
   if (all_h24({&x, &y})) return run_reduce(b, (OpCdotNormH{x, y}), nsites(x), out, 3, st, dres);
-  DISPATCH(x.nr, any64({&x, &y}),
-           return run_reduce(b, (OpCdotNorm<NR, T>{x, y}), nsites(x), out, 3, st, dres));
+  DISPATCH(x, kind({&x, &y}),
+           return run_reduce(b, (OpCdotNorm<NR, T>{x, y}), NS, out, 3, st, dres));
 }
 int blas_caxpy_norm(Blas* b, Cf a, const FieldRef& x, const FieldRef& y, double* out, cudaStream_t st,
                     double* dres) {
   if (all_h24({&x, &y})) return run_reduce(b, (OpCaxpyNormH<false>{x, y, y, a}), nsites(y), out, 1, st, dres);
-  DISPATCH(y.nr, any64({&x, &y}),
-           return run_reduce(b, (OpCaxpyNorm<NR, T, false>{x, y, y, a}), nsites(y), out, 1, st, dres));
+  DISPATCH(y, kind({&x, &y}),
+           return run_reduce(b, (OpCaxpyNorm<NR, T, false>{x, y, y, a}), NS, out, 1, st, dres));
 }
 int blas_caxpy_norm_dot(Blas* b, Cf a, const FieldRef& x, const FieldRef& y, const FieldRef& w,
                         double out[3], cudaStream_t st, double* dres) {
   if (all_h24({&x, &y, &w})) return run_reduce(b, (OpCaxpyNormH<true>{x, y, w, a}), nsites(y), out, 3, st, dres);
-  DISPATCH(y.nr, any64({&x, &y, &w}),
-           return run_reduce(b, (OpCaxpyNorm<NR, T, true>{x, y, w, a}), nsites(y), out, 3, st, dres));
+  DISPATCH(y, kind({&x, &y, &w}),
+           return run_reduce(b, (OpCaxpyNorm<NR, T, true>{x, y, w, a}), NS, out, 3, st, dres));
 }
 int blas_bicg_xr(Blas* b, Cf a, const FieldRef& p, Cf bb, const FieldRef& s, Cf c, const FieldRef& t,
                  const FieldRef& xs, const FieldRef& w, double out[3], cudaStream_t st, double* dres) {
   if (all_h24({&p, &s, &t, &w}) && xs.prec != P64 && xs.nr == 24)
     return run_reduce(b, (OpBicgXRH{p, s, t, xs, w, a, bb, c}), nsites(s), out, 3, st, dres);
-  DISPATCH(s.nr, any64({&p, &s, &t, &xs, &w}),
-           return run_reduce(b, (OpBicgXR<NR, T>{p, s, t, xs, w, a, bb, c}), nsites(s), out, 3, st, dres));
+  DISPATCH(s, kind({&p, &s, &t, &xs, &w}),
+           return run_reduce(b, (OpBicgXR<NR, T>{p, s, t, xs, w, a, bb, c}), NS, out, 3, st, dres));
 }
 int blas_cg_update(Blas* b, Cf a, const FieldRef& p, Cf c, const FieldRef& Ap, const FieldRef& xs,
                    const FieldRef& r, double* out, cudaStream_t st, double* dres) {
-  DISPATCH(r.nr, any64({&p, &Ap, &xs, &r}),
-           return run_reduce(b, (OpCgUpdate<NR, T>{p, Ap, xs, r, a, c}), nsites(r), out, 1, st, dres));
+  DISPATCH(r, kind({&p, &Ap, &xs, &r}),
+           return run_reduce(b, (OpCgUpdate<NR, T>{p, Ap, xs, r, a, c}), NS, out, 1, st, dres));
 }
 int blas_scale_cdot(Blas* b, Cf s, const FieldRef& x, const FieldRef& y, double out[2], cudaStream_t st,
                     double* dres) {
   if (all_h24({&x, &y})) return run_reduce(b, (OpScaleCdotH{x, y, s}), nsites(x), out, 2, st, dres);
-  DISPATCH(x.nr, any64({&x, &y}),
-           return run_reduce(b, (OpScaleCdot<NR, T>{x, y, s}), nsites(x), out, 2, st, dres));
+  DISPATCH(x, kind({&x, &y}),
+           return run_reduce(b, (OpScaleCdot<NR, T>{x, y, s}), NS, out, 2, st, dres));
 }
 int blas_xmy_norm(Blas* b, const FieldRef& bb, const FieldRef& y, double* out, cudaStream_t st, double* dres) {
-  DISPATCH(y.nr, any64({&bb, &y}),
-           return run_reduce(b, (OpXmyNorm<NR, T>{bb, y}), nsites(y), out, 1, st, dres));
+  DISPATCH(y, kind({&bb, &y}),
+           return run_reduce(b, (OpXmyNorm<NR, T>{bb, y}), NS, out, 1, st, dres));
 }
 int blas_multishift_update(Blas* b, int n, const FieldRef* xs, const FieldRef* ps, const FieldRef& r,
                            const double* coef, cudaStream_t st) {
@@ -803,13 +847,14 @@ int blas_multishift_update(Blas* b, int n, const FieldRef* xs, const FieldRef* p
   }
   ShiftFields f;
   f.n = n;
-  bool dbl = r.prec == P64;
+  int kd = kind({&r});
   for (int j = 0; j < n; ++j) {
     f.x[j] = xs[j];
     f.p[j] = ps[j];
-    dbl = dbl || xs[j].prec == P64 || ps[j].prec == P64;
+    const int kj = kind({&xs[j], &ps[j]});
+    if (kj != kd) kd = SOME64;  // two of them differ: FP64 is among them
   }
-  DISPATCH(r.nr, dbl, return run_map(b, (OpMultiShift<NR, T>{f, r, coef}), nsites(r), st));
+  DISPATCH(r, kd, return run_map(b, (OpMultiShift<NR, T>{f, r, coef}), NS, st));
 }
 
 int blas_multi_caxpy(Blas* b, int n, const Cf* c, const FieldRef* xs, const FieldRef& y, cudaStream_t st) {
@@ -822,12 +867,16 @@ int blas_multi_caxpy(Blas* b, int n, const Cf* c, const FieldRef* xs, const Fiel
       m.c[j] = c[j0 + j];
       xdbl = xdbl || xs[j0 + j].prec == P64;
     }
-    int rc;
+    int rc = DIRAC_OK;
     if (y.prec == P64 && !xdbl) {
       if (y.nr == 24) rc = run_map(b, (OpMultiCaxpy<24, double, float>{m, y}), nsites(y), st);
       else rc = run_map(b, (OpMultiCaxpy<6, double, float>{m, y}), nsites(y), st);
     } else {
-      DISPATCH(y.nr, xdbl || y.prec == P64, rc = run_map(b, (OpMultiCaxpy<NR, T, T>{m, y}), nsites(y), st));
+      int kd = kind({&y});
+      for (int j = 0; j < m.n; ++j)
+        if (kind({&m.x[j]}) != kd) kd = SOME64;
+      auto run = [&]() -> int { DISPATCH(y, kd, return run_map(b, (OpMultiCaxpy<NR, T, T>{m, y}), NS, st)); };
+      rc = run();
     }
     if (rc) return rc;
   }
