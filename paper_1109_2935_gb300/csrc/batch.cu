@@ -43,13 +43,9 @@ struct BatchLat {
   int mstride;
 };
 
+// output site idx of right-hand side rhs
 template <int PREC, int R>
-__device__ __forceinline__ void batch_tile(const BatchLat& L, int t, int RG) {
-  const int rgroups_site = L.tiles_site;
-  const int rg = t / rgroups_site, sg = t - rg * rgroups_site;
-  const int rhs = rg * RG + threadIdx.y;
-  if (rhs >= L.nrhs) return;
-  if (L.mask && L.mask[(size_t)(L.rhs0 + rhs) * L.mstride] == 0.0) return;
+__device__ __forceinline__ void batch_site(const BatchLat& L, int rhs, int idx) {
   WilsonArg a;
   a.g = L.g;
   a.gauge = L.gauge;
@@ -64,7 +60,17 @@ __device__ __forceinline__ void batch_tile(const BatchLat& L, int t, int RG) {
   a.in[1] = in + hb;
   a.out[0] = out;
   a.out[1] = out + hb;
-  wilson_site<PREC, R, true>(a, sg * kTileSites + threadIdx.x);
+  wilson_site<PREC, R, true>(a, idx);
+}
+
+template <int PREC, int R>
+__device__ __forceinline__ void batch_tile(const BatchLat& L, int t, int RG) {
+  const int rgroups_site = L.tiles_site;
+  const int rg = t / rgroups_site, sg = t - rg * rgroups_site;
+  const int rhs = rg * RG + threadIdx.y;
+  if (rhs >= L.nrhs) return;
+  if (L.mask && L.mask[(size_t)(L.rhs0 + rhs) * L.mstride] == 0.0) return;
+  batch_site<PREC, R>(L, rhs, sg * kTileSites + threadIdx.x);
 }
 
 // one lattice, descriptor by value
@@ -82,6 +88,69 @@ __global__ void __launch_bounds__(kTileSites * kMaxRG, 1)
     while (l + 1 < nlat && t >= lats[l + 1].tile_begin) ++l;
     const BatchLat L = lats[l];
     batch_tile<PREC, R>(L, t - L.tile_begin, RG);
+  }
+}
+
+// FP64 fields: a warp per (right-hand side, 32-site group), over the right-hand sides that
+// the masks leave. The FP64 pipe bounds this kernel (19 cycles per warp instruction and SM,
+// four schedulers at 64), links and clover come from L2 at a tenth of its rate, so what
+// counts is that every scheduler has the same number of warps with work: with warp y of a
+// CTA tied to right-hand side 4 k + y, a reliable update of a few systems ran on one or two
+// of the four schedulers.
+static constexpr int kBatch64PerSM = 3;
+static constexpr int kMaxBatch64Rhs = 1024;  // right-hand sides listed at a time
+template <int R>
+__global__ void __launch_bounds__(128, kBatch64PerSM)
+    batch_kernel64(const BatchLat* __restrict__ lats, int nlat, int nrhs) {
+  __shared__ int first[kMaxBatch64Rhs + 1];  // first warp item of each listed right-hand side
+  __shared__ int lat[kMaxBatch64Rhs], loc[kMaxBatch64Rhs];
+  __shared__ int listed;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int r0 = 0; r0 < nrhs; r0 += kMaxBatch64Rhs) {
+    const int r1 = min(nrhs, r0 + kMaxBatch64Rhs);
+    __syncthreads();
+    if (w == 0) {
+      int n = 0, items = 0;
+      for (int q0 = r0; q0 < r1; q0 += 32) {
+        const int q = q0 + lane;
+        int l = 0, cnt = 0;
+        if (q < r1) {
+          while (l + 1 < nlat && q >= lats[l + 1].rhs0) ++l;
+          const BatchLat& L = lats[l];
+          if (!L.mask || L.mask[(size_t)q * L.mstride] != 0.0) cnt = L.tiles_site;
+        }
+        const unsigned on = __ballot_sync(0xffffffffu, cnt > 0);
+        int sum = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(0xffffffffu, sum, o);
+          if (lane >= o) sum += t;
+        }
+        if (cnt > 0) {
+          const int k = n + __popc(on & ((1u << lane) - 1));
+          first[k] = items + sum - cnt;
+          lat[k] = l;
+          loc[k] = q - lats[l].rhs0;
+        }
+        n += __popc(on);
+        items += __shfl_sync(0xffffffffu, sum, 31);
+      }
+      if (lane == 0) {
+        listed = n;
+        first[n] = items;
+      }
+    }
+    __syncthreads();
+    const int n = listed, items = first[n];
+    for (int i = blockIdx.x * 4 + w; i < items; i += gridDim.x * 4) {
+      int a = 0, b = n;  // first[a] <= i < first[b]
+      while (b - a > 1) {
+        const int m = (a + b) >> 1;
+        if (first[m] <= i) a = m;
+        else b = m;
+      }
+      batch_site<P64, R>(lats[lat[a]], loc[a], (i - first[a]) * kTileSites + lane);
+    }
   }
 }
 
@@ -111,6 +180,12 @@ static void launch_batch_prec(int recon, const BatchLat* d, int nlat, int ntiles
   if (recon == 18) batch_kernel<PREC, 18><<<grid, block, 0, st>>>(d, nlat, ntiles, RG);
   else if (recon == 12) batch_kernel<PREC, 12><<<grid, block, 0, st>>>(d, nlat, ntiles, RG);
   else batch_kernel<PREC, 8><<<grid, block, 0, st>>>(d, nlat, ntiles, RG);
+}
+
+static void launch_batch64(int recon, const BatchLat* d, int nlat, int nrhs, int grid, cudaStream_t st) {
+  if (recon == 18) batch_kernel64<18><<<grid, 128, 0, st>>>(d, nlat, nrhs);
+  else if (recon == 12) batch_kernel64<12><<<grid, 128, 0, st>>>(d, nlat, nrhs);
+  else batch_kernel64<8><<<grid, 128, 0, st>>>(d, nlat, nrhs);
 }
 
 static BatchLat describe(const dirac_ctx* c, int prec, const void* in, void* out, int nrhs, int RG) {
@@ -157,7 +232,7 @@ struct dirac_batch {
   std::vector<dirac_ctx*> ctxs;
   std::vector<BatchLat> lats;    // host copy (RG-dependent fields refreshed by the tuner)
   BatchLat* d_lats = nullptr;    // device table
-  int prec = 0, recon = 12, ntiles = 0;
+  int prec = 0, recon = 12, ntiles = 0, nrhs = 0;
   bool ds = false;               // FP64 fields: double-single arithmetic (18-real links)
   int RG = 1, per_sm = 1, grid = 1;
   double tuned_ms = 0;
@@ -207,7 +282,7 @@ static void batch_launch_direct(dirac_batch* b, cudaStream_t st) {
   }
   if (b->prec == P64 && b->ds)
     batch_kernel_ds<<<b->grid, dim3(kTileSites, 4), 0, st>>>(b->d_lats, nlat, b->ntiles);
-  else if (b->prec == P64) launch_batch_prec<P64>(b->recon, b->d_lats, nlat, b->ntiles, b->RG, b->grid, st);
+  else if (b->prec == P64) launch_batch64(b->recon, b->d_lats, nlat, b->nrhs, b->grid, st);
   else if (b->prec == P32) launch_batch_prec<P32>(b->recon, b->d_lats, nlat, b->ntiles, b->RG, b->grid, st);
   else launch_batch_prec<P16>(b->recon, b->d_lats, nlat, b->ntiles, b->RG, b->grid, st);
 }
@@ -271,7 +346,10 @@ int batch_create(dirac_ctx* const* ctxs, int nlat, void* const* out, const void*
     b->lats.push_back(describe(ctxs[l], prec, in[l], out[l], nrhs[l], 1));
     b->lats.back().rhs0 = r0;
     r0 += nrhs[l];
+    b->nrhs = r0;
   }
+  // FP64 fields have one kernel and one shape (batch_kernel64)
+  const bool k64 = prec == P64 && !ds;
   if (cudaMalloc(&b->d_lats, sizeof(BatchLat) * nlat) != cudaSuccess) {
     cudaGetLastError();
     delete b;
@@ -292,7 +370,7 @@ int batch_create(dirac_ctx* const* ctxs, int nlat, void* const* out, const void*
     const int RG = kCand[k][0], per_sm = kCand[k][1];
     // tune < 2: only the shape (4 right-hand sides per CTA, 4 CTAs per SM)
     // (the default shape also serves plans with fewer right-hand sides: idle warps exit)
-    if ((tune == 2 && RG > max_rhs && RG > 1) || (tune < 2 && k != kDefaultCand)) {
+    if (tune < 2 || k64 ? k != kDefaultCand : RG > max_rhs && RG > 1) {
       b->cand_ms.push_back(-1);
       continue;
     }
@@ -304,7 +382,7 @@ int batch_create(dirac_ctx* const* ctxs, int nlat, void* const* out, const void*
     }
     b->RG = RG;
     if (batch_layout(b, RG, st)) break;
-    b->grid = grid_for(per_sm, b->ntiles);
+    b->grid = grid_for(k64 ? kBatch64PerSM : per_sm, b->ntiles);
     batch_launch_direct(b, st);
     cudaEventRecord(e0, st);
     for (int r = 0; r < 3; ++r) batch_launch_direct(b, st);
@@ -327,7 +405,7 @@ int batch_create(dirac_ctx* const* ctxs, int nlat, void* const* out, const void*
     return DIRAC_ERR_CUDA;
   }
   b->RG = kCand[bi][0];
-  b->per_sm = kCand[bi][1];
+  b->per_sm = k64 ? kBatch64PerSM : kCand[bi][1];
   if (batch_layout(b, b->RG, st)) {
     cudaFree(b->d_lats);
     delete b;

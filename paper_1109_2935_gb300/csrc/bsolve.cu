@@ -267,27 +267,37 @@ template <int SP, int AP> struct OpRestart {  // rs = r (sloppy); xs = 0
 };
 
 // ---------------------------------------------------------------- kernels
-__device__ __forceinline__ void block_sum(double v[3], int n) {
-  __shared__ double sh[NT / 32][3];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int k = 0; k < n; ++k) {
-    double x = v[k];
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (lane == 0) sh[w][k] = x;
-  }
+// Sums of NRED values over a block into sum[] of shared memory: warp k adds value k (FP64
+// instructions issue at one per 64 cycles and scheduler, so few and parallel chains count).
+template <int NRED> struct RedShared {
+  double v[NRED][NT];
+  double sum[NRED];
+  bool last;
+};
+template <int NRED>
+__device__ __forceinline__ void block_sum(const double* acc, RedShared<NRED>& sh) {
+  const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+#pragma unroll
+  for (int j = 0; j < NRED; ++j) sh.v[j][threadIdx.x] = acc[j];
   __syncthreads();
-  if (threadIdx.x == 0)
-    for (int k = 0; k < n; ++k) {
-      double x = 0;
-      for (int j = 0; j < NT / 32; ++j) x += sh[j][k];
-      v[k] = x;
-    }
+  if (k < NRED) {
+    double t[NT / 32];
+#pragma unroll
+    for (int j = 0; j < NT / 32; ++j) t[j] = sh.v[k][lane + 32 * j];
+#pragma unroll
+    for (int w = NT / 64; w > 0; w >>= 1)
+#pragma unroll
+      for (int j = 0; j < w; ++j) t[j] += t[j + w];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t[0] += __shfl_xor_sync(0xffffffffu, t[0], o);
+    if (lane == 0) sh.sum[k] = t[0];
+  }
   __syncthreads();
 }
 
 // One launch over every right-hand side of every segment: block b -> (segment,
 // right-hand side, block within it). Reductions: per right-hand side, each block writes
-// its partial sums; the last block of that right-hand side adds them in block order
+// its partial sums; the last block of that right-hand side adds them in a fixed order
 // (deterministic) into its scalar slots.
 // A right-hand side whose mask entry (mask[rhs * mstride], when mask is given) is 0 is
 // skipped by all its blocks: no site work, no partial sums, its ticket untouched.
@@ -306,24 +316,24 @@ __global__ void __launch_bounds__(NT) mb_kernel(const Seg* __restrict__ segs, in
   const int n = 2 * g.Vh;
   for (int s = bx * NT + threadIdx.x; s < n; s += g.bpr * NT) op(g, r, s, sc, acc);
   if constexpr (Op::NRED > 0) {
-    __shared__ bool last;
-    block_sum(acc, Op::NRED);
+    __shared__ RedShared<Op::NRED> sh;
+    block_sum<Op::NRED>(acc, sh);
     if (threadIdx.x == 0) {
       double* pp = part + ((size_t)rhs * MAXBPR + bx) * 3;
-      for (int j = 0; j < Op::NRED; ++j) pp[j] = acc[j];
+      for (int j = 0; j < Op::NRED; ++j) pp[j] = sh.sum[j];
       __threadfence();
-      last = atomicAdd(tick + rhs, 1u) == (unsigned)g.bpr - 1;
+      sh.last = atomicAdd(tick + rhs, 1u) == (unsigned)g.bpr - 1;
     }
     __syncthreads();
-    if (!last) return;
+    if (!sh.last) return;
     __threadfence();
-    if (threadIdx.x == 0) {
-      double s3[3] = {0, 0, 0};
-      for (int b = 0; b < g.bpr; ++b)
-        for (int j = 0; j < Op::NRED; ++j) s3[j] += __ldcg(part + ((size_t)rhs * MAXBPR + b) * 3 + j);
-      for (int j = 0; j < Op::NRED; ++j) sc[Op::OUT + j] = s3[j];
-      tick[rhs] = 0;
-    }
+    static_assert(MAXBPR <= NT, "one partial sum per thread");
+    const bool mine = (int)threadIdx.x < g.bpr;
+    for (int j = 0; j < Op::NRED; ++j)
+      acc[j] = mine ? __ldcg(part + ((size_t)rhs * MAXBPR + threadIdx.x) * 3 + j) : 0.0;
+    block_sum<Op::NRED>(acc, sh);
+    if (threadIdx.x < Op::NRED) sc[Op::OUT + threadIdx.x] = sh.sum[threadIdx.x];
+    if (threadIdx.x == 0) tick[rhs] = 0;
   }
 }
 
@@ -762,7 +772,9 @@ extern "C" int solve_batched(dirac_ctx* const* ctxs, int nlat, void* const* x, c
     g.nrhs = nrhs[l];
     g.rhs0 = rhs0;
     g.blk0 = blk;
-    long bpr = (2 * c->Vh + NT * 16 - 1) / (NT * 16);
+    // two sites per thread up to MAXBPR blocks: a launch often covers few of the systems
+    // (those that take a reliable update), whose blocks alone have to fill the chip
+    long bpr = (2 * c->Vh + NT * 2 - 1) / (NT * 2);
     g.bpr = (int)(bpr < 1 ? 1 : (bpr > MAXBPR ? MAXBPR : bpr));
     for (int v = 0; v < NVEC; ++v) {
       g.fb[v] = 2 * spinor_half_bytes(prec_of[v], 24, c->Vh);
