@@ -265,6 +265,7 @@ int dirac_create(const dirac_params* params, dirac_ctx** out) {
   c->Vh = V / 2;
   c->g.Vh = (int)c->Vh;
   c->g.apbc = p.t_antiperiodic ? 1 : 0;
+  geom_divisors(c->g);
   c->nr = p.kind == DIRAC_WILSON_CLOVER ? 24 : 6;
   c->mask = mask;
   c->blas = blas_create();

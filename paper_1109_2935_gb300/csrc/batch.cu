@@ -35,7 +35,7 @@ struct BatchLat {
   char* out;
   size_t field_bytes;
   int nrhs;
-  int tiles_site;       // 32-site groups over the 2 Vh output sites
+  int tiles_site;       // 32-site groups (of one parity) of the lattice
   int tiles;            // tiles_site * ceil(nrhs / RG)
   int tile_begin;       // first tile of this lattice in the batch
   int rhs0;             // plan-wide index of this lattice's first right-hand side
@@ -43,8 +43,8 @@ struct BatchLat {
   int mstride;
 };
 
-// output site idx of right-hand side rhs
-template <int PREC, int R>
+// output site idx of right-hand sides rhs .. rhs + N - 1
+template <int PREC, int R, int N = 1>
 __device__ __forceinline__ void batch_site(const BatchLat& L, int rhs, int idx) {
   WilsonArg a;
   a.g = L.g;
@@ -60,34 +60,50 @@ __device__ __forceinline__ void batch_site(const BatchLat& L, int rhs, int idx) 
   a.in[1] = in + hb;
   a.out[0] = out;
   a.out[1] = out + hb;
-  wilson_site<PREC, R, true>(a, idx);
+  wilson_site<PREC, R, true, N>(a, idx, L.field_bytes);
 }
 
-template <int PREC, int R>
+// Tile t of lattice L: warp y of the CTA has right-hand sides y NR .. y NR + NR - 1 of the
+// tile's RG (warp-uniform, so that the fields are uniform addresses). Where one of a pair
+// is missing or masked out, the other runs alone.
+template <int PREC, int R, int NR>
 __device__ __forceinline__ void batch_tile(const BatchLat& L, int t, int RG) {
-  const int rgroups_site = L.tiles_site;
-  const int rg = t / rgroups_site, sg = t - rg * rgroups_site;
-  const int rhs = rg * RG + threadIdx.y;
-  if (rhs >= L.nrhs) return;
-  if (L.mask && L.mask[(size_t)(L.rhs0 + rhs) * L.mstride] == 0.0) return;
-  batch_site<PREC, R>(L, rhs, sg * kTileSites + threadIdx.x);
+  const int rg = t / L.tiles_site, sg = t - rg * L.tiles_site;
+  const int y = __shfl_sync(0xffffffffu, threadIdx.y, 0);
+  int rhs = rg * RG + y * NR;
+  const int idx = sg * kTileSites + threadIdx.x;
+  auto on = [&](int r) { return r < L.nrhs && !(L.mask && L.mask[(size_t)(L.rhs0 + r) * L.mstride] == 0.0); };
+  const bool first = on(rhs);
+  if constexpr (NR == 2) {
+    const bool second = on(rhs + 1);
+    if (first && second) {
+      batch_site<PREC, R, 2>(L, rhs, idx);
+      return;
+    }
+    if (!first && !second) return;
+    if (!first) ++rhs;
+  } else {
+    if (!first) return;
+  }
+  batch_site<PREC, R, 1>(L, rhs, idx);
 }
 
 // one lattice, descriptor by value
-template <int PREC, int R>
-__global__ void __launch_bounds__(kTileSites * kMaxRG, 1) mrhs_kernel(const BatchLat L, int RG) {
-  for (int t = blockIdx.x; t < L.tiles; t += gridDim.x) batch_tile<PREC, R>(L, t, RG);
+template <int PREC, int R, int NR>
+__global__ void __launch_bounds__(kTileSites * kMaxRG, 1) mrhs_kernel(const __grid_constant__ BatchLat L, int RG) {
+  for (int t = blockIdx.x; t < L.tiles; t += gridDim.x) batch_tile<PREC, R, NR>(L, t, RG);
 }
 
-// several lattices: descriptor table in device memory, tiles numbered across lattices
-template <int PREC, int R>
+// several lattices: descriptor table in the parameter space (uniform loads), tiles numbered
+// across lattices
+struct LatTable { BatchLat v[kMaxLat]; };
+template <int PREC, int R, int NR>
 __global__ void __launch_bounds__(kTileSites * kMaxRG, 1)
-    batch_kernel(const BatchLat* __restrict__ lats, int nlat, int ntiles, int RG) {
+    batch_kernel(const __grid_constant__ LatTable lats, int nlat, int ntiles, int RG) {
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
     int l = 0;
-    while (l + 1 < nlat && t >= lats[l + 1].tile_begin) ++l;
-    const BatchLat L = lats[l];
-    batch_tile<PREC, R>(L, t - L.tile_begin, RG);
+    while (l + 1 < nlat && t >= lats.v[l + 1].tile_begin) ++l;
+    batch_tile<PREC, R, NR>(lats.v[l], t - lats.v[l].tile_begin, RG);
   }
 }
 
@@ -162,24 +178,26 @@ __global__ void __launch_bounds__(kTileSites * 4, 1)
     int l = 0;
     while (l + 1 < nlat && t >= lats[l + 1].tile_begin) ++l;
     const BatchLat L = lats[l];
-    batch_tile<P64DS, 18>(L, t - L.tile_begin, 4);
+    batch_tile<P64DS, 18, 1>(L, t - L.tile_begin, 4);
   }
 }
 
-template <int PREC>
+template <int PREC, int NR>
 static void launch_mrhs_prec(int recon, const BatchLat& L, int RG, int grid, cudaStream_t st) {
-  dim3 block(kTileSites, RG);
-  if (recon == 18) mrhs_kernel<PREC, 18><<<grid, block, 0, st>>>(L, RG);
-  else if (recon == 12) mrhs_kernel<PREC, 12><<<grid, block, 0, st>>>(L, RG);
-  else mrhs_kernel<PREC, 8><<<grid, block, 0, st>>>(L, RG);
+  dim3 block(kTileSites, RG / NR);
+  if (recon == 18) mrhs_kernel<PREC, 18, NR><<<grid, block, 0, st>>>(L, RG);
+  else if (recon == 12) mrhs_kernel<PREC, 12, NR><<<grid, block, 0, st>>>(L, RG);
+  else mrhs_kernel<PREC, 8, NR><<<grid, block, 0, st>>>(L, RG);
 }
-template <int PREC>
-static void launch_batch_prec(int recon, const BatchLat* d, int nlat, int ntiles, int RG, int grid,
-                              cudaStream_t st) {
-  dim3 block(kTileSites, RG);
-  if (recon == 18) batch_kernel<PREC, 18><<<grid, block, 0, st>>>(d, nlat, ntiles, RG);
-  else if (recon == 12) batch_kernel<PREC, 12><<<grid, block, 0, st>>>(d, nlat, ntiles, RG);
-  else batch_kernel<PREC, 8><<<grid, block, 0, st>>>(d, nlat, ntiles, RG);
+template <int PREC, int NR>
+static void launch_batch_prec(int recon, const std::vector<BatchLat>& l, int ntiles, int RG, int grid, cudaStream_t st) {
+  LatTable t;
+  for (size_t k = 0; k < l.size(); ++k) t.v[k] = l[k];
+  const int nlat = (int)l.size();
+  dim3 block(kTileSites, RG / NR);
+  if (recon == 18) batch_kernel<PREC, 18, NR><<<grid, block, 0, st>>>(t, nlat, ntiles, RG);
+  else if (recon == 12) batch_kernel<PREC, 12, NR><<<grid, block, 0, st>>>(t, nlat, ntiles, RG);
+  else batch_kernel<PREC, 8, NR><<<grid, block, 0, st>>>(t, nlat, ntiles, RG);
 }
 
 static void launch_batch64(int recon, const BatchLat* d, int nlat, int nrhs, int grid, cudaStream_t st) {
@@ -198,7 +216,7 @@ static BatchLat describe(const dirac_ctx* c, int prec, const void* in, void* out
   L.out = (char*)out;
   L.field_bytes = 2 * spinor_half_bytes(prec, 24, c->Vh);
   L.nrhs = nrhs;
-  L.tiles_site = (int)((2 * c->Vh + kTileSites - 1) / kTileSites);
+  L.tiles_site = full_sites((int)c->Vh) / kTileSites;
   L.tiles = L.tiles_site * ((nrhs + RG - 1) / RG);
   L.tile_begin = 0;
   L.rhs0 = 0;
@@ -234,7 +252,7 @@ struct dirac_batch {
   BatchLat* d_lats = nullptr;    // device table
   int prec = 0, recon = 12, ntiles = 0, nrhs = 0;
   bool ds = false;               // FP64 fields: double-single arithmetic (18-real links)
-  int RG = 1, per_sm = 1, grid = 1;
+  int RG = 1, NR = 1, per_sm = 1, grid = 1;
   double tuned_ms = 0;
   std::vector<double> cand_ms;   // autotuner timings, candidate order
   cudaGraph_t graph = nullptr;
@@ -251,9 +269,34 @@ struct dirac_batch {
 
 namespace dirac {
 
-// the tile-shape candidates: (right-hand sides per CTA, resident CTAs per SM)
-static const int kCand[][2] = {{1, 16}, {2, 8}, {4, 4}, {8, 2}, {16, 1}, {2, 16}, {4, 8}, {8, 4}};
-static constexpr int kDefaultCand = 2;  // the shape the full tuning picks on the batched workloads
+// the tile-shape candidates: (right-hand sides per CTA, resident CTAs per SM, right-hand
+// sides per thread); all fill the 16 warps per SM of the 128-register cap
+static const int kCand[][3] = {{1, 16, 1}, {2, 8, 1}, {4, 4, 1}, {8, 2, 1}, {2, 16, 2}, {4, 8, 2}, {8, 4, 2}};
+static constexpr int kDefaultCand = 2, kDefaultPair = 5;
+
+// Two right-hand sides per thread load and rebuild every link once for both, but a thread
+// takes about 1.6 times as long and there are half as many: worth it from about two waves of
+// resident warps on (16 per SM). Measured, one right-hand side per thread -> two, us: FP32
+// 12^3x20 x 7 26.8 -> 22.9, 16^4 x 12 102.6 -> 80.8, 16^3x32 x 2 33.0 -> 29.2, 8^4 x 12 8.6 ->
+// 9.1; FP16 16^4 x 12 80.2 -> 66.0, 16^3x32 x 7 84.0 -> 89.3, 12^3x20 x 12 38.6 -> 37.1, 8^3x16
+// x 7 8.8 -> 10.2. With an odd count one thread of each group has a single right-hand side,
+// which FP16 (compute-bound) does not make up for.
+static bool pair_rhs(int prec, long groups, int nrhs) {
+  if (prec == P64 || groups * nrhs <= 32l * sm_count()) return false;
+  return nrhs % 2 == 0 || (prec == P32 && nrhs >= 5);
+}
+
+// Warps per CTA for `items` warps on the same sites: the most (up to 4, they share the links
+// through L1) of those that leave the fewest of an SM's 16 warps idle. (12 warps of 12 right-
+// hand sides left a quarter of the SM empty: FP32 16^4 x 12 took 102.6 us against 51.6 x 7.)
+static int group_warps(int items) {
+  int best = 1, busy = 0;
+  for (int w = 1; w <= 4; ++w) {
+    const int b = 1000 * items / ((items + w - 1) / w * w) * (16 / w * w);
+    if (b >= busy) busy = b, best = w;
+  }
+  return best;
+}
 
 static int batch_layout(dirac_batch* b, int RG, cudaStream_t st) {
   int begin = 0;
@@ -283,8 +326,8 @@ static void batch_launch_direct(dirac_batch* b, cudaStream_t st) {
   if (b->prec == P64 && b->ds)
     batch_kernel_ds<<<b->grid, dim3(kTileSites, 4), 0, st>>>(b->d_lats, nlat, b->ntiles);
   else if (b->prec == P64) launch_batch64(b->recon, b->d_lats, nlat, b->nrhs, b->grid, st);
-  else if (b->prec == P32) launch_batch_prec<P32>(b->recon, b->d_lats, nlat, b->ntiles, b->RG, b->grid, st);
-  else launch_batch_prec<P16>(b->recon, b->d_lats, nlat, b->ntiles, b->RG, b->grid, st);
+  else if (b->prec == P32) (b->NR == 2 ? launch_batch_prec<P32, 2> : launch_batch_prec<P32, 1>)(b->recon, b->lats, b->ntiles, b->RG, b->grid, st);
+  else (b->NR == 2 ? launch_batch_prec<P16, 2> : launch_batch_prec<P16, 1>)(b->recon, b->lats, b->ntiles, b->RG, b->grid, st);
 }
 
 }  // namespace dirac
@@ -300,14 +343,14 @@ int dirac_apply_multi(dirac_ctx* c, void* out, const void* in, int nrhs, dirac_p
   const size_t fb = 2 * spinor_half_bytes(prec, 24, c->Vh);
   const char *i0 = (const char*)in, *o0 = (const char*)out;
   if (i0 < o0 + fb * nrhs && o0 < i0 + fb * nrhs) return set_err(c, DIRAC_ERR_ARG, "in and out overlap");
-  const int RG = nrhs < kMaxRG ? nrhs : kMaxRG;
-  BatchLat L = describe(c, prec, in, out, nrhs, RG);
-  const int per_sm = kMaxRG / RG;  // 16 resident warps per SM at the 128-register cap
-  const int grid = grid_for(per_sm, L.tiles);
+  const int NR = pair_rhs(prec, full_sites((int)c->Vh) / kTileSites, nrhs) ? 2 : 1;
+  const int warps = group_warps((nrhs + NR - 1) / NR), RG = warps * NR;
+  const BatchLat L = describe(c, prec, in, out, nrhs, RG);
+  const int grid = grid_for(16 / warps, L.tiles);
   cudaStream_t st = (cudaStream_t)stream;
-  if ((int)prec == P64) launch_mrhs_prec<P64>(c->p.recon[prec], L, RG, grid, st);
-  else if ((int)prec == P32) launch_mrhs_prec<P32>(c->p.recon[prec], L, RG, grid, st);
-  else launch_mrhs_prec<P16>(c->p.recon[prec], L, RG, grid, st);
+  if ((int)prec == P64) launch_mrhs_prec<P64, 1>(c->p.recon[prec], L, RG, grid, st);
+  else if ((int)prec == P32) (NR == 2 ? launch_mrhs_prec<P32, 2> : launch_mrhs_prec<P32, 1>)(c->p.recon[prec], L, RG, grid, st);
+  else (NR == 2 ? launch_mrhs_prec<P16, 2> : launch_mrhs_prec<P16, 1>)(c->p.recon[prec], L, RG, grid, st);
   return cuda_check(c, "multi-RHS kernel");
 }
 
@@ -365,12 +408,17 @@ int batch_create(dirac_ctx* const* ctxs, int nlat, void* const* out, const void*
   cudaEventCreate(&e1);
   double best = INFINITY;
   int bi = 0;
+  // the untimed shape: pairs if they pay on every lattice
+  bool pairs = true;
+  for (int l = 0; l < nlat; ++l) pairs = pairs && pair_rhs(prec, b->lats[l].tiles_site, nrhs[l]);
+  const int untimed = pairs ? kDefaultPair : kDefaultCand;
   const int ncand = (int)(sizeof(kCand) / sizeof(kCand[0]));
   for (int k = 0; k < ncand; ++k) {
     const int RG = kCand[k][0], per_sm = kCand[k][1];
-    // tune < 2: only the shape (4 right-hand sides per CTA, 4 CTAs per SM)
+    b->NR = kCand[k][2];
+    // tune < 2: only the default shape (4 right-hand sides per CTA)
     // (the default shape also serves plans with fewer right-hand sides: idle warps exit)
-    if (tune < 2 || k64 ? k != kDefaultCand : RG > max_rhs && RG > 1) {
+    if (tune < 2 || k64 ? k != untimed : RG > max_rhs && RG > 1) {
       b->cand_ms.push_back(-1);
       continue;
     }
@@ -405,6 +453,7 @@ int batch_create(dirac_ctx* const* ctxs, int nlat, void* const* out, const void*
     return DIRAC_ERR_CUDA;
   }
   b->RG = kCand[bi][0];
+  b->NR = kCand[bi][2];
   b->per_sm = k64 ? kBatch64PerSM : kCand[bi][1];
   if (batch_layout(b, b->RG, st)) {
     cudaFree(b->d_lats);

@@ -26,20 +26,52 @@ struct Geom {
   int Lxh;       // LX / 2
   int Vh;        // sites per parity
   int apbc;      // antiperiodic t for fermion hops
+  // division of a site index by Lxh, LY, LZ: n / d = (n m >> 32) >> s, exact for n < 2^31
+  // (m = ceil(2^p / d), p = 31 + ceil(log2 d): the error of m times n stays below 2^p);
+  // m = 0 stands for d = 1. A runtime division costs about 20 instructions, three of them
+  // a twentieth of a stencil thread.
+  unsigned m[3], s[3];
 };
+
+inline void geom_divisors(Geom& g) {
+  const int d[3] = {g.Lxh, g.L[1], g.L[2]};
+  for (int k = 0; k < 3; ++k) {
+    g.m[k] = g.s[k] = 0;
+    if (d[k] <= 1) continue;
+    int c = 0;
+    while ((1ll << c) < d[k]) ++c;
+    g.m[k] = (unsigned)(((1ull << (31 + c)) + d[k] - 1) / (unsigned)d[k]);
+    g.s[k] = c - 1;
+  }
+}
+
+__device__ __forceinline__ int geom_div(const Geom& g, int k, int n) {
+  return g.m[k] ? (int)(__umulhi((unsigned)n, g.m[k]) >> g.s[k]) : n;
+}
 
 // Coordinates of checkerboard site cb of parity par.
 __device__ __forceinline__ void cb_coords(const Geom& g, int cb, int par, int x[4]) {
-  int xh = cb % g.Lxh;
-  int r = cb / g.Lxh;
-  x[1] = r % g.L[1]; r /= g.L[1];
-  x[2] = r % g.L[2];
-  x[3] = r / g.L[2];
+  const int r = geom_div(g, 0, cb), q = geom_div(g, 1, r);
+  const int xh = cb - r * g.Lxh;
+  x[1] = r - q * g.L[1];
+  x[3] = geom_div(g, 2, q);
+  x[2] = q - x[3] * g.L[2];
   x[0] = 2 * xh + ((par + x[1] + x[2] + x[3]) & 1);
 }
 
 __device__ __forceinline__ int cb_index(const Geom& g, const int x[4]) {
   return ((x[3] * g.L[2] + x[2]) * g.L[1] + x[1]) * g.Lxh + (x[0] >> 1);
+}
+
+// Checkerboard index (of the other parity) of the neighbour of site (x, cb) in direction
+// mu; edge: the hop wraps around the lattice.
+__device__ __forceinline__ int hop_index(const Geom& g, const int x[4], int cb, int mu, bool fwd, bool& edge) {
+  const int last = g.L[mu] - 1, v = x[mu];
+  edge = fwd ? v == last : v == 0;
+  const int y = fwd ? (edge ? 0 : v + 1) : (edge ? last : v - 1);
+  if (mu == 0) return cb + (y >> 1) - (v >> 1);
+  const int stride = mu == 1 ? g.Lxh : mu == 2 ? g.Lxh * g.L[1] : g.Lxh * g.L[1] * g.L[2];
+  return cb + (y - v) * stride;
 }
 
 // ---------------------------------------------------------------- complex helpers
@@ -99,6 +131,36 @@ __device__ __forceinline__ void su3_mv_dag(const Link<T>& U, const C<T> h[3], C<
   }
 }
 
+// Two complex numbers side by side in the lanes of packed FP32 instructions (add / mul /
+// fma .f32x2, each lane rounded as the scalar instruction): one issue slot for two results.
+struct C2 { float2 r, i; };
+__device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ C2 pair2(C<float> a, C<float> b) {
+  return C2{make_float2(a.r, b.r), make_float2(a.i, b.i)};
+}
+// v = U h (DAG: U^dagger h) for two 3-vectors with the same link
+template <bool DAG>
+__device__ __forceinline__ void su3_mv2(const Link<float>& U, const C2 h[3], C2 v[3]) {
+  float2 n[3];  // the factor that enters with a minus sign
+#pragma unroll
+  for (int b = 0; b < 3; ++b) n[b] = neg2(DAG ? h[b].r : h[b].i);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    float2 r, i;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const C<float> u = DAG ? U.m[b][a] : U.m[a][b];
+      const float2 ur = dup2(u.r), ui = dup2(u.i);
+      r = b ? __ffma2_rn(ur, h[b].r, r) : __fmul2_rn(ur, h[b].r);
+      i = b ? __ffma2_rn(ur, h[b].i, i) : __fmul2_rn(ur, h[b].i);
+      r = __ffma2_rn(ui, DAG ? h[b].i : n[b], r);
+      i = __ffma2_rn(ui, DAG ? n[b] : h[b].r, i);
+    }
+    v[a] = C2{r, i};
+  }
+}
+
 // fma of one binary16 half of word a and one of word b into an FP32 accumulator: the two
 // binary16 factors enter the fused multiply-add exactly (their product is exact in FP32),
 // so this equals converting both and one FP32 fma, without the conversions.
@@ -114,6 +176,11 @@ __device__ __forceinline__ float fma_hh(uint32_t a, uint32_t b, float c) {
 }
 
 // ---------------------------------------------------------------- raw chunk I/O
+// Chunk k of site cb in an array of BYTES-byte chunks, Vh per plane: the plane's address is
+// the same for every thread of a warp, the site's offset the same for every plane.
+template <int BYTES> __device__ __forceinline__ const char* chunk_at(const char* b, int k, int Vh, int cb) {
+  return b + (size_t)k * Vh * BYTES + (size_t)(unsigned)cb * BYTES;
+}
 template <typename V> __device__ __forceinline__ V ldg_chunk(const char* p) {
   return __ldg(reinterpret_cast<const V*>(p));
 }
@@ -150,14 +217,14 @@ template <int NR> struct SpinorIO<P64, NR> {
   __device__ static void load(const char* b, int Vh, int cb, double v[NR]) {
 #pragma unroll
     for (int k = 0; k < NR / 2; ++k) {
-      double2 q = ld_chunk<double2, NC>(b + ((size_t)k * Vh + cb) * 16);
+      double2 q = ld_chunk<double2, NC>(chunk_at<16>(b, k, Vh, cb));
       v[2 * k] = q.x; v[2 * k + 1] = q.y;
     }
   }
   __device__ static void store(char* b, int Vh, int cb, const double v[NR]) {
 #pragma unroll
     for (int k = 0; k < NR / 2; ++k)
-      *reinterpret_cast<double2*>(b + ((size_t)k * Vh + cb) * 16) = make_double2(v[2 * k], v[2 * k + 1]);
+      *reinterpret_cast<double2*>(const_cast<char*>(chunk_at<16>(b, k, Vh, cb))) = make_double2(v[2 * k], v[2 * k + 1]);
   }
 };
 
@@ -167,14 +234,14 @@ template <> struct SpinorIO<P32, 24> {
   __device__ static void load(const char* b, int Vh, int cb, float v[24]) {
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-      float4 q = ld_chunk<float4, NC>(b + ((size_t)k * Vh + cb) * 16);
+      float4 q = ld_chunk<float4, NC>(chunk_at<16>(b, k, Vh, cb));
       v[4 * k] = q.x; v[4 * k + 1] = q.y; v[4 * k + 2] = q.z; v[4 * k + 3] = q.w;
     }
   }
   __device__ static void store(char* b, int Vh, int cb, const float v[24]) {
 #pragma unroll
     for (int k = 0; k < 6; ++k)
-      *reinterpret_cast<float4*>(b + ((size_t)k * Vh + cb) * 16) =
+      *reinterpret_cast<float4*>(const_cast<char*>(chunk_at<16>(b, k, Vh, cb))) =
           make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
   }
 };
@@ -185,14 +252,14 @@ template <> struct SpinorIO<P32, 6> {
   __device__ static void load(const char* b, int Vh, int cb, float v[6]) {
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      float2 q = ld_chunk<float2, NC>(b + ((size_t)k * Vh + cb) * 8);
+      float2 q = ld_chunk<float2, NC>(chunk_at<8>(b, k, Vh, cb));
       v[2 * k] = q.x; v[2 * k + 1] = q.y;
     }
   }
   __device__ static void store(char* b, int Vh, int cb, const float v[6]) {
 #pragma unroll
     for (int k = 0; k < 3; ++k)
-      *reinterpret_cast<float2*>(b + ((size_t)k * Vh + cb) * 8) = make_float2(v[2 * k], v[2 * k + 1]);
+      *reinterpret_cast<float2*>(const_cast<char*>(chunk_at<8>(b, k, Vh, cb))) = make_float2(v[2 * k], v[2 * k + 1]);
   }
 };
 
@@ -210,7 +277,7 @@ template <> struct SpinorIO<P16, 24> {
   __device__ static float load_raw(const char* b, int Vh, int cb, float v[24]) {
     const float n = ld_chunk<float, NC>(b + (size_t)48 * Vh + (size_t)cb * 4);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) unpack_half8(ld_chunk<int4, NC>(b + ((size_t)k * Vh + cb) * 16), v + 8 * k);
+    for (int k = 0; k < 3; ++k) unpack_half8(ld_chunk<int4, NC>(chunk_at<16>(b, k, Vh, cb)), v + 8 * k);
     return n;
   }
   template <bool NC = true>
@@ -218,7 +285,7 @@ template <> struct SpinorIO<P16, 24> {
     float n = ld_chunk<float, NC>(b + (size_t)48 * Vh + (size_t)cb * 4);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      int4 q = ld_chunk<int4, NC>(b + ((size_t)k * Vh + cb) * 16);
+      int4 q = ld_chunk<int4, NC>(chunk_at<16>(b, k, Vh, cb));
       unpack_half8(q, v + 8 * k);
     }
 #pragma unroll
@@ -231,7 +298,7 @@ template <> struct SpinorIO<P16, 24> {
     for (int k = 0; k < 24; ++k) w[k] = v[k] * inv;
 #pragma unroll
     for (int k = 0; k < 3; ++k)
-      *reinterpret_cast<int4*>(b + ((size_t)k * Vh + cb) * 16) = pack_half8(w + 8 * k);
+      *reinterpret_cast<int4*>(const_cast<char*>(chunk_at<16>(b, k, Vh, cb))) = pack_half8(w + 8 * k);
     reinterpret_cast<float*>(b + (size_t)48 * Vh)[cb] = n;
   }
 };
@@ -244,7 +311,7 @@ template <> struct SpinorIO<P16, 6> {
     const float n = ld_chunk<float, NC>(b + (size_t)12 * Vh + (size_t)cb * 4);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const float2 q = __half22float2(ld_chunk<__half2, NC>(b + ((size_t)k * Vh + cb) * 4));
+      const float2 q = __half22float2(ld_chunk<__half2, NC>(chunk_at<4>(b, k, Vh, cb)));
       v[2 * k] = q.x; v[2 * k + 1] = q.y;
     }
     return n;
@@ -254,7 +321,7 @@ template <> struct SpinorIO<P16, 6> {
     float n = ld_chunk<float, NC>(b + (size_t)12 * Vh + (size_t)cb * 4);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      __half2 q = ld_chunk<__half2, NC>(b + ((size_t)k * Vh + cb) * 4);
+      __half2 q = ld_chunk<__half2, NC>(chunk_at<4>(b, k, Vh, cb));
       float2 f = __half22float2(q);
       v[2 * k] = f.x * n; v[2 * k + 1] = f.y * n;
     }
@@ -264,7 +331,7 @@ template <> struct SpinorIO<P16, 6> {
     float n = site_norm_scale(v, 6, inv);
 #pragma unroll
     for (int k = 0; k < 3; ++k)
-      *reinterpret_cast<__half2*>(b + ((size_t)k * Vh + cb) * 4) =
+      *reinterpret_cast<__half2*>(const_cast<char*>(chunk_at<4>(b, k, Vh, cb))) =
           __floats2half2_rn(v[2 * k] * inv, v[2 * k + 1] * inv);
     reinterpret_cast<float*>(b + (size_t)12 * Vh)[cb] = n;
   }
@@ -343,20 +410,20 @@ struct LinkIO {
     if constexpr (PREC == P64) {
 #pragma unroll
       for (int k = 0; k < R / 2; ++k) {
-        double2 q = ld_chunk<double2, NC>(plane + ((size_t)k * stride + i) * 16);
+        double2 q = ld_chunk<double2, NC>(chunk_at<16>(plane, k, stride, i));
         v[2 * k] = (T)q.x; v[2 * k + 1] = (T)q.y;
       }
     } else if constexpr (PREC == P32) {
       if constexpr (R == 18) {
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-          float2 q = ld_chunk<float2, NC>(plane + ((size_t)k * stride + i) * 8);
+          float2 q = ld_chunk<float2, NC>(chunk_at<8>(plane, k, stride, i));
           v[2 * k] = q.x; v[2 * k + 1] = q.y;
         }
       } else {
 #pragma unroll
         for (int k = 0; k < R / 4; ++k) {
-          float4 q = ld_chunk<float4, NC>(plane + ((size_t)k * stride + i) * 16);
+          float4 q = ld_chunk<float4, NC>(chunk_at<16>(plane, k, stride, i));
           v[4 * k] = q.x; v[4 * k + 1] = q.y; v[4 * k + 2] = q.z; v[4 * k + 3] = q.w;
         }
       }
@@ -364,13 +431,13 @@ struct LinkIO {
       if constexpr (R == 18) {
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
-          float2 f = __half22float2(ld_chunk<__half2, NC>(plane + ((size_t)k * stride + i) * 4));
+          float2 f = __half22float2(ld_chunk<__half2, NC>(chunk_at<4>(plane, k, stride, i)));
           v[2 * k] = f.x; v[2 * k + 1] = f.y;
         }
       } else if constexpr (R == 12) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          uint2 q = ld_chunk<uint2, NC>(plane + ((size_t)k * stride + i) * 8);
+          uint2 q = ld_chunk<uint2, NC>(chunk_at<8>(plane, k, stride, i));
           const __half2* h = reinterpret_cast<const __half2*>(&q);
           float2 f0 = __half22float2(h[0]), f1 = __half22float2(h[1]);
           v[4 * k] = f0.x; v[4 * k + 1] = f0.y; v[4 * k + 2] = f1.x; v[4 * k + 3] = f1.y;
@@ -410,20 +477,20 @@ struct LinkIO {
     }
     if constexpr (PREC == P64) {
       for (int k = 0; k < R / 2; ++k)
-        *reinterpret_cast<double2*>(plane + ((size_t)k * Vh + cb) * 16) = make_double2(v[2 * k], v[2 * k + 1]);
+        *reinterpret_cast<double2*>(const_cast<char*>(chunk_at<16>(plane, k, Vh, cb))) = make_double2(v[2 * k], v[2 * k + 1]);
     } else if constexpr (PREC == P32) {
       if constexpr (R == 18) {
         for (int k = 0; k < 9; ++k)
-          *reinterpret_cast<float2*>(plane + ((size_t)k * Vh + cb) * 8) = make_float2((float)v[2 * k], (float)v[2 * k + 1]);
+          *reinterpret_cast<float2*>(const_cast<char*>(chunk_at<8>(plane, k, Vh, cb))) = make_float2((float)v[2 * k], (float)v[2 * k + 1]);
       } else {
         for (int k = 0; k < R / 4; ++k)
-          *reinterpret_cast<float4*>(plane + ((size_t)k * Vh + cb) * 16) =
+          *reinterpret_cast<float4*>(const_cast<char*>(chunk_at<16>(plane, k, Vh, cb))) =
               make_float4((float)v[4 * k], (float)v[4 * k + 1], (float)v[4 * k + 2], (float)v[4 * k + 3]);
       }
     } else {
       if constexpr (R == 18) {
         for (int k = 0; k < 9; ++k)
-          *reinterpret_cast<__half2*>(plane + ((size_t)k * Vh + cb) * 4) =
+          *reinterpret_cast<__half2*>(const_cast<char*>(chunk_at<4>(plane, k, Vh, cb))) =
               __floats2half2_rn((float)v[2 * k], (float)v[2 * k + 1]);
       } else if constexpr (R == 12) {
         for (int k = 0; k < 3; ++k) {
@@ -431,7 +498,7 @@ struct LinkIO {
           __half2* h = reinterpret_cast<__half2*>(&q);
           h[0] = __floats2half2_rn((float)v[4 * k], (float)v[4 * k + 1]);
           h[1] = __floats2half2_rn((float)v[4 * k + 2], (float)v[4 * k + 3]);
-          *reinterpret_cast<uint2*>(plane + ((size_t)k * Vh + cb) * 8) = q;
+          *reinterpret_cast<uint2*>(const_cast<char*>(chunk_at<8>(plane, k, Vh, cb))) = q;
         }
       } else {
         float f[8];
@@ -454,13 +521,13 @@ template <> struct CloverIO<P64> {
   __device__ static void load(const char* b, int Vh, int cb, double v[72]) {
 #pragma unroll
     for (int k = 0; k < 36; ++k) {
-      double2 q = ldg_chunk<double2>(b + ((size_t)k * Vh + cb) * 16);
+      double2 q = ldg_chunk<double2>(chunk_at<16>(b, k, Vh, cb));
       v[2 * k] = q.x; v[2 * k + 1] = q.y;
     }
   }
   __device__ static void store(char* b, int Vh, int cb, const double v[72]) {
     for (int k = 0; k < 36; ++k)
-      *reinterpret_cast<double2*>(b + ((size_t)k * Vh + cb) * 16) = make_double2(v[2 * k], v[2 * k + 1]);
+      *reinterpret_cast<double2*>(const_cast<char*>(chunk_at<16>(b, k, Vh, cb))) = make_double2(v[2 * k], v[2 * k + 1]);
   }
 };
 template <> struct CloverIO<P32> {
@@ -468,13 +535,13 @@ template <> struct CloverIO<P32> {
   __device__ static void load(const char* b, int Vh, int cb, float v[72]) {
 #pragma unroll
     for (int k = 0; k < 18; ++k) {
-      float4 q = ldg_chunk<float4>(b + ((size_t)k * Vh + cb) * 16);
+      float4 q = ldg_chunk<float4>(chunk_at<16>(b, k, Vh, cb));
       v[4 * k] = q.x; v[4 * k + 1] = q.y; v[4 * k + 2] = q.z; v[4 * k + 3] = q.w;
     }
   }
   __device__ static void store(char* b, int Vh, int cb, const double v[72]) {
     for (int k = 0; k < 18; ++k)
-      *reinterpret_cast<float4*>(b + ((size_t)k * Vh + cb) * 16) =
+      *reinterpret_cast<float4*>(const_cast<char*>(chunk_at<16>(b, k, Vh, cb))) =
           make_float4((float)v[4 * k], (float)v[4 * k + 1], (float)v[4 * k + 2], (float)v[4 * k + 3]);
   }
 };
@@ -484,13 +551,13 @@ template <> struct CloverIO<P16> {
   __device__ static float load_raw(const char* b, int Vh, int cb, float v[72]) {
     const float n = __ldg(reinterpret_cast<const float*>(b + (size_t)144 * Vh) + cb);
 #pragma unroll
-    for (int k = 0; k < 9; ++k) unpack_half8(ldg_chunk<int4>(b + ((size_t)k * Vh + cb) * 16), v + 8 * k);
+    for (int k = 0; k < 9; ++k) unpack_half8(ldg_chunk<int4>(chunk_at<16>(b, k, Vh, cb)), v + 8 * k);
     return n;
   }
   __device__ static void load(const char* b, int Vh, int cb, float v[72]) {
     float n = __ldg(reinterpret_cast<const float*>(b + (size_t)144 * Vh) + cb);
 #pragma unroll
-    for (int k = 0; k < 9; ++k) unpack_half8(ldg_chunk<int4>(b + ((size_t)k * Vh + cb) * 16), v + 8 * k);
+    for (int k = 0; k < 9; ++k) unpack_half8(ldg_chunk<int4>(chunk_at<16>(b, k, Vh, cb)), v + 8 * k);
 #pragma unroll
     for (int k = 0; k < 72; ++k) v[k] *= n;
   }
@@ -501,7 +568,7 @@ template <> struct CloverIO<P16> {
     for (int k = 0; k < 9; ++k) {
       float f[8];
       for (int j = 0; j < 8; ++j) f[j] = (float)v[8 * k + j] * inv;
-      *reinterpret_cast<int4*>(b + ((size_t)k * Vh + cb) * 16) = pack_half8(f);
+      *reinterpret_cast<int4*>(const_cast<char*>(chunk_at<16>(b, k, Vh, cb))) = pack_half8(f);
     }
     reinterpret_cast<float*>(b + (size_t)144 * Vh)[cb] = m;
   }
@@ -514,13 +581,13 @@ __device__ __forceinline__ void clover_block(const char* b, int stride, int i, i
   if constexpr (PREC == P64) {
 #pragma unroll
     for (int k = 0; k < 18; ++k) {
-      double2 q = ld_chunk<double2, NC>(b + ((size_t)(18 * blk + k) * stride + i) * 16);
+      double2 q = ld_chunk<double2, NC>(chunk_at<16>(b, (18 * blk + k), stride, i));
       v[2 * k] = (T)q.x; v[2 * k + 1] = (T)q.y;
     }
   } else if constexpr (PREC == P32) {
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-      float4 q = ld_chunk<float4, NC>(b + ((size_t)(9 * blk + k) * stride + i) * 16);
+      float4 q = ld_chunk<float4, NC>(chunk_at<16>(b, (9 * blk + k), stride, i));
       v[4 * k] = q.x; v[4 * k + 1] = q.y; v[4 * k + 2] = q.z; v[4 * k + 3] = q.w;
     }
   } else {
@@ -528,7 +595,7 @@ __device__ __forceinline__ void clover_block(const char* b, int stride, int i, i
     const float n = ld_chunk<float, NC>(b + (size_t)144 * stride + (size_t)i * 4);
     float f[40];
 #pragma unroll
-    for (int k = 0; k < 5; ++k) unpack_half8(ld_chunk<int4, NC>(b + ((size_t)(4 * blk + k) * stride + i) * 16), f + 8 * k);
+    for (int k = 0; k < 5; ++k) unpack_half8(ld_chunk<int4, NC>(chunk_at<16>(b, (4 * blk + k), stride, i)), f + 8 * k);
     const int off = 4 * blk;  // block 1 starts 4 halves into chunk 4
 #pragma unroll
     for (int k = 0; k < 36; ++k) v[k] = f[k + off] * n;

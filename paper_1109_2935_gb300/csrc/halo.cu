@@ -423,6 +423,7 @@ extern "C" int dirac_dd_create_grid(dirac_ctx* c, const int* grid, dirac_prec pr
   }
   d->gl.Lxh = d->gl.L[0] / 2;
   d->gl.Vh = c->g.Vh / P;
+  geom_divisors(d->gl);
   for (int mu = 0; mu < 4; ++mu) d->F[mu] = face_volume(d->gl, mu);
   d->r.resize(P);
   for (int q = 0; q < P; ++q) {

@@ -74,12 +74,57 @@ __device__ __forceinline__ void wilson_project(const T* psi, T s, C<T> h0[3], C<
   }
 }
 
+// wilson_hop_proj in FP32: the two spin components of the half spinor meet the same link,
+// so they ride in the two lanes of packed instructions (the same roundings, fewer issue
+// slots: FP16 M at 24^3x128 141 -> 137 us, FP32 M 192 -> 190 us).
+template <int MU>
+__device__ __forceinline__ void wilson_hop_pair(C<float> acc[4][3], const C<float> h0[3], const C<float> h1[3],
+                                                const Link<float>& U, bool link_dag, float s, float bc) {
+  C2 h[3], v[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) h[c] = pair2(h0[c], h1[c]);
+  if (link_dag) su3_mv2<true>(U, h, v);
+  else su3_mv2<false>(U, h, v);
+  const float ks = s * bc;
+  const float2 b2 = dup2(bc), k2 = dup2(ks), x2 = make_float2(ks, -ks), y2 = make_float2(-ks, ks);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    C2 up = pair2(acc[0][c], acc[1][c]);
+    up.r = __ffma2_rn(b2, v[c].r, up.r);
+    up.i = __ffma2_rn(b2, v[c].i, up.i);
+    acc[0][c] = C<float>{up.r.x, up.i.x};
+    acc[1][c] = C<float>{up.r.y, up.i.y};
+    if (MU == 0) {        // B^dagger v = (-i v1, -i v0)
+      acc[2][c] = C<float>{fmaf(ks, v[c].i.y, acc[2][c].r), fmaf(-ks, v[c].r.y, acc[2][c].i)};
+      acc[3][c] = C<float>{fmaf(ks, v[c].i.x, acc[3][c].r), fmaf(-ks, v[c].r.x, acc[3][c].i)};
+    } else if (MU == 1) { // B^dagger v = (v1, -v0)
+      acc[2][c] = C<float>{fmaf(ks, v[c].r.y, acc[2][c].r), fmaf(ks, v[c].i.y, acc[2][c].i)};
+      acc[3][c] = C<float>{fmaf(-ks, v[c].r.x, acc[3][c].r), fmaf(-ks, v[c].i.x, acc[3][c].i)};
+    } else {
+      C2 lo = pair2(acc[2][c], acc[3][c]);
+      if (MU == 2) {      // B^dagger v = (-i v0, i v1)
+        lo.r = __ffma2_rn(x2, v[c].i, lo.r);
+        lo.i = __ffma2_rn(y2, v[c].r, lo.i);
+      } else {
+        lo.r = __ffma2_rn(k2, v[c].r, lo.r);
+        lo.i = __ffma2_rn(k2, v[c].i, lo.i);
+      }
+      acc[2][c] = C<float>{lo.r.x, lo.i.x};
+      acc[3][c] = C<float>{lo.r.y, lo.i.y};
+    }
+  }
+}
+
 // The rest of a hop after the projection: v = U h (U^dagger h for a backward hop), then
 // acc += bc P-reconstruction of v.
 template <int MU, typename T>
 __device__ __forceinline__ void wilson_hop_proj(C<T> acc[4][3], const C<T> h0[3], const C<T> h1[3],
                                                 const Link<T>& U, bool link_dag, T s, T bc) {
   C<T> v0[3], v1[3];
+  if constexpr (std::is_same<T, float>::value) {
+    wilson_hop_pair<MU>(acc, h0, h1, U, link_dag, s, bc);
+    return;
+  }
   if (link_dag) {
     su3_mv_dag(U, h0, v0);
     su3_mv_dag(U, h1, v1);
@@ -129,7 +174,7 @@ __device__ __forceinline__ void apply_clover_site(const char* b, int Vh, int cb,
       T v[36];
 #pragma unroll
       for (int k = 0; k < 18; ++k) {
-        double2 q = ldg_chunk<double2>(b + ((size_t)(18 * blk + k) * Vh + cb) * 16);
+        double2 q = ldg_chunk<double2>(chunk_at<16>(b, (18 * blk + k), Vh, cb));
         v[2 * k] = T(q.x); v[2 * k + 1] = T(q.y);
       }
       herm6_mv<T>(v, in + 6 * blk, out + 6 * blk);
@@ -140,7 +185,7 @@ __device__ __forceinline__ void apply_clover_site(const char* b, int Vh, int cb,
       float v[36];
 #pragma unroll
       for (int k = 0; k < 9; ++k) {
-        float4 q = ldg_chunk<float4>(b + ((size_t)(9 * blk + k) * Vh + cb) * 16);
+        float4 q = ldg_chunk<float4>(chunk_at<16>(b, (9 * blk + k), Vh, cb));
         v[4 * k] = q.x; v[4 * k + 1] = q.y; v[4 * k + 2] = q.z; v[4 * k + 3] = q.w;
       }
       herm6_mv<T>(v, in + 6 * blk, out + 6 * blk);
@@ -196,14 +241,14 @@ __device__ __forceinline__ void clover_self_h(const char* clov, const char* self
   uint32_t x[12];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const int4 q = ldg_chunk<int4>(self + ((size_t)k * Vh + cb) * 16);
+    const int4 q = ldg_chunk<int4>(chunk_at<16>(self, k, Vh, cb));
     x[4 * k] = (uint32_t)q.x; x[4 * k + 1] = (uint32_t)q.y; x[4 * k + 2] = (uint32_t)q.z; x[4 * k + 3] = (uint32_t)q.w;
   }
   // block 0: words 0..17 (chunks 0..3 and half of chunk 4); block 1: words 18..35
   uint32_t c[20];
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
-    const int4 q = ldg_chunk<int4>(clov + ((size_t)k * Vh + cb) * 16);
+    const int4 q = ldg_chunk<int4>(chunk_at<16>(clov, k, Vh, cb));
     c[4 * k] = (uint32_t)q.x; c[4 * k + 1] = (uint32_t)q.y; c[4 * k + 2] = (uint32_t)q.z; c[4 * k + 3] = (uint32_t)q.w;
   }
   herm6_hh(c, x, av);
@@ -211,7 +256,7 @@ __device__ __forceinline__ void clover_self_h(const char* clov, const char* self
   c[1] = c[19];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const int4 q = ldg_chunk<int4>(clov + ((size_t)(5 + k) * Vh + cb) * 16);
+    const int4 q = ldg_chunk<int4>(chunk_at<16>(clov, (5 + k), Vh, cb));
     c[2 + 4 * k] = (uint32_t)q.x; c[3 + 4 * k] = (uint32_t)q.y; c[4 + 4 * k] = (uint32_t)q.z; c[5 + 4 * k] = (uint32_t)q.w;
   }
   herm6_hh(c, x + 6, av + 6);
@@ -225,11 +270,11 @@ __device__ __forceinline__ void clover_self_h(const char* clov, const char* self
 // reals), the lower two kept as binary16 pairs (l, 6 words: spin 2 colours 0..2, spin 3
 // colours 0..2, re low / im high); returns bc times the site norm, the hop's factor.
 __device__ __forceinline__ float load_hop_h(const char* src, int Vh, int cb, float u[12], uint32_t l[6], float bc) {
-  const float n = __ldg(reinterpret_cast<const float*>(src + (size_t)48 * Vh) + cb);
+  const float n = __ldg(reinterpret_cast<const float*>(chunk_at<4>(src, 12, Vh, cb)));
   uint32_t w[12];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const int4 q = ldg_chunk<int4>(src + ((size_t)k * Vh + cb) * 16);
+    const int4 q = ldg_chunk<int4>(chunk_at<16>(src, k, Vh, cb));
     w[4 * k] = (uint32_t)q.x; w[4 * k + 1] = (uint32_t)q.y; w[4 * k + 2] = (uint32_t)q.z; w[4 * k + 3] = (uint32_t)q.w;
   }
 #pragma unroll
@@ -280,50 +325,128 @@ __device__ __forceinline__ void wilson_hop_h(C<float> acc[4][3], const float u[1
 // Launch shape per storage precision (threads per CTA, minimum resident CTAs per SM,
 // which caps registers). FP32/FP16 are memory-latency bound and want many warps in
 // flight; FP64 is FP64-ALU bound on this part.
-#ifndef WILSON_INTERLEAVE
-#define WILSON_INTERLEAVE 32
-#endif
-// Measured on GB300 at 24^3x128 (clover M): FP32 64x8 (128-register cap) 0.199 ms vs
+// Measured on GB300 at 24^3x128 (clover M, before the packed arithmetic): FP32 64x8 (128-register cap) 0.199 ms vs
 // 128x1 (up to 255 registers) 0.288 ms; FP16 ~0.178 ms for every shape tried.
 template <int PREC> struct WilsonShape { static constexpr int threads = 64, minb = 10; };
 template <> struct WilsonShape<P32> { static constexpr int threads = 64, minb = 8; };
 template <> struct WilsonShape<P64> { static constexpr int threads = 128, minb = 1; };
 template <> struct WilsonShape<P64DS> { static constexpr int threads = 128, minb = 2; };
 
-// Output site idx of the full operator. The two parities alternate every
-// WILSON_INTERLEAVE threads (a warp: the parity stays warp-uniform): the forward link
-// U_mu(x) read by site x is read again as a backward link by the neighbour x + mu of the
-// other parity close in time, so it comes from cache instead of a second DRAM pass over
-// all links.
-__device__ __forceinline__ void full_site(int idx, int Vh, int& par, int& cb) {
-  constexpr int IL = WILSON_INTERLEAVE;
-  const int grp = idx / (2 * IL), k = idx - grp * 2 * IL;
-  if ((grp + 1) * IL <= Vh) {
-    par = k >= IL;
-    cb = grp * IL + k - par * IL;
-  } else {  // last, incomplete pair of groups (Vh not a multiple of IL)
-    const int half = Vh - grp * IL;
-    par = k >= half;
-    cb = grp * IL + k - par * half;
+// Output site idx of the full operator. The two parities alternate every 32 threads (a
+// warp): the forward link U_mu(x) read by site x is read again as a backward link by the
+// neighbour x + mu of the other parity close in time, so it comes from cache instead of a
+// second DRAM pass over all links. The parity is made warp-uniform (all lanes enter), so
+// that the field and link planes of a thread are uniform addresses. full_sites: the number
+// of idx values, idle ones of a ragged last warp (cb >= Vh) included.
+__host__ __device__ __forceinline__ int full_sites(int Vh) { return (Vh + 31) / 32 * 64; }
+__device__ __forceinline__ void full_site(int idx, int& par, int& cb) {
+  const int w = __shfl_sync(0xffffffffu, idx >> 5, 0);
+  par = w & 1;
+  cb = (w >> 1) * 32 + (idx & 31);
+}
+
+// out = Ahat self - kappa acc for N right-hand sides of one site, chirality block by block:
+// a block's clover is loaded once for all of them. acc is overwritten with the result.
+template <int PREC, int N>
+__device__ __forceinline__ void clover_site_n(const char* clov, const char* self, size_t stride, int Vh, int cb,
+                                              float mk, C<float> acc[N][4][3]) {
+#pragma unroll
+  for (int blk = 0; blk < 2; ++blk) {
+    if constexpr (PREC == P16) {
+      uint32_t c[20];
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        const int4 q = ldg_chunk<int4>(chunk_at<16>(clov, 4 * blk + k, Vh, cb));
+        c[4 * k] = (uint32_t)q.x; c[4 * k + 1] = (uint32_t)q.y; c[4 * k + 2] = (uint32_t)q.z; c[4 * k + 3] = (uint32_t)q.w;
+      }
+      const float nc = __ldg(reinterpret_cast<const float*>(chunk_at<4>(clov, 36, Vh, cb)));
+#pragma unroll
+      for (int r = 0; r < N; ++r) {
+        const char* s = self + r * stride;
+        uint32_t x[8];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const int4 q = ldg_chunk<int4>(chunk_at<16>(s, blk + k, Vh, cb));
+          x[4 * k] = (uint32_t)q.x; x[4 * k + 1] = (uint32_t)q.y; x[4 * k + 2] = (uint32_t)q.z; x[4 * k + 3] = (uint32_t)q.w;
+        }
+        const float n = nc * __ldg(reinterpret_cast<const float*>(chunk_at<4>(s, 12, Vh, cb)));
+        C<float> y[6];
+        herm6_hh(c + 2 * blk, x + 2 * blk, y);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+          C<float>& o = acc[r][2 * blk + k / 3][k % 3];
+          o = C<float>{fmaf(mk, o.r, n * y[k].r), fmaf(mk, o.i, n * y[k].i)};
+        }
+      }
+    } else {
+      float v[36];
+#pragma unroll
+      for (int k = 0; k < 9; ++k) {
+        const float4 q = ldg_chunk<float4>(chunk_at<16>(clov, 9 * blk + k, Vh, cb));
+        v[4 * k] = q.x; v[4 * k + 1] = q.y; v[4 * k + 2] = q.z; v[4 * k + 3] = q.w;
+      }
+#pragma unroll
+      for (int r = 0; r < N; ++r) {
+        C<float> x[6], y[6];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const float4 q = ldg_chunk<float4>(chunk_at<16>(self + r * stride, 3 * blk + k, Vh, cb));
+          x[2 * k] = C<float>{q.x, q.y};
+          x[2 * k + 1] = C<float>{q.z, q.w};
+        }
+        herm6_mv<float>(v, x, y);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+          C<float>& o = acc[r][2 * blk + k / 3][k % 3];
+          o = C<float>{fmaf(mk, o.r, y[k].r), fmaf(mk, o.i, y[k].i)};
+        }
+      }
+    }
   }
 }
 
-// One output site of the stencil: thread index idx over the Vh (hop mode) or 2 Vh
-// (full operator) output sites. Shared by the single-RHS, multi-RHS and batched kernels.
-template <int PREC, int R, bool FULLM>
-__device__ __forceinline__ void wilson_site(const WilsonArg& a, int idx) {
+// One hop for N right-hand sides: the link is loaded and rebuilt once.
+template <int PREC, int R, int N, int MU, typename T>
+__device__ __forceinline__ void wilson_hop_n(C<T> acc[N][4][3], const char* src, size_t stride, const char* gauge,
+                                             int Vh, int ycb, int lpar, int lcb, bool dag, T s, T bc) {
+  if constexpr (PREC == P16) {
+    float u[N][12], n[N];
+    uint32_t l[N][6];
+#pragma unroll
+    for (int r = 0; r < N; ++r) n[r] = load_hop_h(src + r * stride, Vh, ycb, u[r], l[r], bc);
+    Link<T> U;
+    LinkIO<PREC, R>::load(gauge, Vh, MU, lpar, lcb, U);
+#pragma unroll
+    for (int r = 0; r < N; ++r) wilson_hop_h<MU>(acc[r], u[r], l[r], U, dag, s, n[r]);
+  } else {
+    T psi[N][24], n[N];
+#pragma unroll
+    for (int r = 0; r < N; ++r) n[r] = load_hop_spinor<PREC, T>(src + r * stride, Vh, ycb, psi[r], bc);
+    Link<T> U;
+    LinkIO<PREC, R>::load(gauge, Vh, MU, lpar, lcb, U);
+#pragma unroll
+    for (int r = 0; r < N; ++r) wilson_hop<MU>(acc[r], psi[r], U, dag, s, n[r]);
+  }
+}
+
+// One output site of the stencil: thread index idx over the Vh (hop mode) or full_sites
+// (full operator) indices. Shared by the single-RHS, multi-RHS and batched kernels. N > 1
+// (FP32 / FP16 full operator): N right-hand sides, `stride` bytes apart, with one load and
+// rebuild of every link and one load of the clover; each gets the bits of N = 1.
+template <int PREC, int R, bool FULLM, int N = 1>
+__device__ __forceinline__ void wilson_site(const WilsonArg& a, int idx, size_t stride = 0) {
   using T = typename Real<PREC>::T;
+  static_assert(N == 1 || (FULLM && (PREC == P32 || PREC == P16)), "");
   const Geom& g = a.g;
   const int Vh = g.Vh;
   int par, cb;
   if (FULLM) {
-    if (idx >= 2 * Vh) return;
-    full_site(idx, Vh, par, cb);
+    full_site(idx, par, cb);
   } else {
-    if (idx >= Vh) return;
     par = a.out_parity;
     cb = idx;
   }
+  if (cb >= Vh) return;
   int x[4];
   cb_coords(g, cb, par, x);
   // selects, not a runtime index into the parameter arrays (which would copy them
@@ -334,95 +457,58 @@ __device__ __forceinline__ void wilson_site(const WilsonArg& a, int idx) {
   const T sf = a.dagger ? (T)1 : (T)-1;  // forward projector 1 - gamma (adjoint: 1 + gamma)
   const T sb = -sf;
 
-  C<T> acc[4][3];
+  C<T> acc[N][4][3];
 #pragma unroll
-  for (int s = 0; s < 4; ++s)
+  for (int r = 0; r < N; ++r)
 #pragma unroll
-    for (int c = 0; c < 3; ++c) acc[s][c] = C<T>{0, 0};
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) acc[r][s][c] = C<T>{0, 0};
 
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) {
     if (!FULLM && a.s == 0.0) break;  // hop mode without the hopping term
-    // forward neighbour x + mu, link U_mu(x) stored at (mu, par, cb)
-    {
-      int y[4] = {x[0], x[1], x[2], x[3]};
-      T bc = 1;
-      if (++y[mu] == g.L[mu]) {
-        y[mu] = 0;
-        if (mu == 3 && g.apbc) bc = -1;
-      }
-      if constexpr (PREC == P16) {
-        float u[12];
-        uint32_t l[6];
-        bc = load_hop_h(src, Vh, cb_index(g, y), u, l, bc);
-        Link<T> U;
-        LinkIO<PREC, R>::load(a.gauge, Vh, mu, par, cb, U);
-        if (mu == 0) wilson_hop_h<0>(acc, u, l, U, false, sf, bc);
-        if (mu == 1) wilson_hop_h<1>(acc, u, l, U, false, sf, bc);
-        if (mu == 2) wilson_hop_h<2>(acc, u, l, U, false, sf, bc);
-        if (mu == 3) wilson_hop_h<3>(acc, u, l, U, false, sf, bc);
-      } else {
-        T psi[24];
-        bc = load_hop_spinor<PREC, T>(src, Vh, cb_index(g, y), psi, bc);
-        Link<T> U;
-        LinkIO<PREC, R>::load(a.gauge, Vh, mu, par, cb, U);
-        if (mu == 0) wilson_hop<0>(acc, psi, U, false, sf, bc);
-        if (mu == 1) wilson_hop<1>(acc, psi, U, false, sf, bc);
-        if (mu == 2) wilson_hop<2>(acc, psi, U, false, sf, bc);
-        if (mu == 3) wilson_hop<3>(acc, psi, U, false, sf, bc);
-      }
-    }
-    // backward neighbour x - mu, link U_mu(x - mu) stored at (mu, 1 - par, cb(x - mu))
-    {
-      int y[4] = {x[0], x[1], x[2], x[3]};
-      T bc = 1;
-      if (y[mu]-- == 0) {
-        y[mu] = g.L[mu] - 1;
-        if (mu == 3 && g.apbc) bc = -1;
-      }
-      int ycb = cb_index(g, y);
-      if constexpr (PREC == P16) {
-        float u[12];
-        uint32_t l[6];
-        bc = load_hop_h(src, Vh, ycb, u, l, bc);
-        Link<T> U;
-        LinkIO<PREC, R>::load(a.gauge, Vh, mu, 1 - par, ycb, U);
-        if (mu == 0) wilson_hop_h<0>(acc, u, l, U, true, sb, bc);
-        if (mu == 1) wilson_hop_h<1>(acc, u, l, U, true, sb, bc);
-        if (mu == 2) wilson_hop_h<2>(acc, u, l, U, true, sb, bc);
-        if (mu == 3) wilson_hop_h<3>(acc, u, l, U, true, sb, bc);
-      } else {
-        T psi[24];
-        bc = load_hop_spinor<PREC, T>(src, Vh, ycb, psi, bc);
-        Link<T> U;
-        LinkIO<PREC, R>::load(a.gauge, Vh, mu, 1 - par, ycb, U);
-        if (mu == 0) wilson_hop<0>(acc, psi, U, true, sb, bc);
-        if (mu == 1) wilson_hop<1>(acc, psi, U, true, sb, bc);
-        if (mu == 2) wilson_hop<2>(acc, psi, U, true, sb, bc);
-        if (mu == 3) wilson_hop<3>(acc, psi, U, true, sb, bc);
-      }
+#pragma unroll
+    for (int dir = 0; dir < 2; ++dir) {
+      // forward neighbour x + mu with link U_mu(x), stored at (mu, par, cb); backward
+      // neighbour x - mu with U_mu(x - mu)^dagger, stored at (mu, 1 - par, cb(x - mu))
+      bool edge;
+      const int ycb = hop_index(g, x, cb, mu, dir == 0, edge);
+      const T bc = (mu == 3 && edge && g.apbc) ? (T)-1 : (T)1;
+      const int lpar = dir ? 1 - par : par, lcb = dir ? ycb : cb;
+      const T s = dir ? sb : sf;
+      if (mu == 0) wilson_hop_n<PREC, R, N, 0, T>(acc, src, stride, a.gauge, Vh, ycb, lpar, lcb, dir == 1, s, bc);
+      if (mu == 1) wilson_hop_n<PREC, R, N, 1, T>(acc, src, stride, a.gauge, Vh, ycb, lpar, lcb, dir == 1, s, bc);
+      if (mu == 2) wilson_hop_n<PREC, R, N, 2, T>(acc, src, stride, a.gauge, Vh, ycb, lpar, lcb, dir == 1, s, bc);
+      if (mu == 3) wilson_hop_n<PREC, R, N, 3, T>(acc, src, stride, a.gauge, Vh, ycb, lpar, lcb, dir == 1, s, bc);
     }
   }
 
   T out[24];
-  bool clover_done = false;
-  if constexpr (FULLM && PREC == P16) {
-    if (a.clover) {  // Ahat self from the stored binary16 values (no conversions)
-      C<float> av[12];
-      clover_self_h(a.clover + (size_t)par * CloverIO<P16>::parity_bytes(Vh), self_in, Vh, cb, av);
-      const float mk = -(float)a.kappa;
+  if constexpr (FULLM && (PREC == P32 || PREC == P16)) {
+    const float mk = -(float)a.kappa;
+    if (a.clover)
+      clover_site_n<PREC, N>(a.clover + (size_t)par * CloverIO<PREC>::parity_bytes(Vh), self_in, stride, Vh, cb, mk, acc);
 #pragma unroll
-      for (int s = 0; s < 4; ++s)
+    for (int r = 0; r < N; ++r) {
+      if (!a.clover) {
+        float self[24];
+        SpinorIO<PREC, 24>::load(self_in + r * stride, Vh, cb, self);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          out[6 * s + 2 * c] = fmaf(mk, acc[s][c].r, av[3 * s + c].r);
-          out[6 * s + 2 * c + 1] = fmaf(mk, acc[s][c].i, av[3 * s + c].i);
+        for (int k = 0; k < 12; ++k) {
+          C<float>& o = acc[r][k / 3][k % 3];
+          o = C<float>{fmaf(mk, o.r, self[2 * k]), fmaf(mk, o.i, self[2 * k + 1])};
         }
-      clover_done = true;
+      }
+#pragma unroll
+      for (int k = 0; k < 12; ++k) {
+        out[2 * k] = acc[r][k / 3][k % 3].r;
+        out[2 * k + 1] = acc[r][k / 3][k % 3].i;
+      }
+      SpinorIO<PREC, 24>::store(dst + r * stride, Vh, cb, out);
     }
-  }
-  if (clover_done) {
-  } else if (FULLM) {
+    return;
+  } else if constexpr (FULLM) {
     T self[24];
     C<T> sv[12], av[12];
     SpinorIO<PREC, 24>::load(self_in, Vh, cb, self);
@@ -439,8 +525,8 @@ __device__ __forceinline__ void wilson_site(const WilsonArg& a, int idx) {
     for (int s = 0; s < 4; ++s)
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        out[6 * s + 2 * c] = fma(mk, acc[s][c].r, av[3 * s + c].r);
-        out[6 * s + 2 * c + 1] = fma(mk, acc[s][c].i, av[3 * s + c].i);
+        out[6 * s + 2 * c] = fma(mk, acc[0][s][c].r, av[3 * s + c].r);
+        out[6 * s + 2 * c + 1] = fma(mk, acc[0][s][c].i, av[3 * s + c].i);
       }
   } else {
     const T sc = (T)a.s;
@@ -448,7 +534,7 @@ __device__ __forceinline__ void wilson_site(const WilsonArg& a, int idx) {
 #pragma unroll
     for (int s = 0; s < 4; ++s)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) v[3 * s + c] = sc * acc[s][c];
+      for (int c = 0; c < 3; ++c) v[3 * s + c] = sc * acc[0][s][c];
     const size_t pb = CloverIO<PREC>::parity_bytes(Vh);
     if (a.self) {
       C<T> cv[12];
@@ -498,7 +584,7 @@ __global__ void __launch_bounds__(WilsonShape<PREC>::threads, WilsonShape<PREC>:
 
 template <int PREC>
 void launch_wilson_prec(int recon, bool fullm, const WilsonArg& a, cudaStream_t st) {
-  int n = fullm ? 2 * a.g.Vh : a.g.Vh;
+  const int n = fullm ? full_sites(a.g.Vh) : a.g.Vh;
   constexpr int T = WilsonShape<PREC>::threads;
   dim3 block(T), grid((n + T - 1) / T);
   if (recon == 18) {

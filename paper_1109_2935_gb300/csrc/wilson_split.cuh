@@ -49,7 +49,10 @@ __global__ void __launch_bounds__(32) wilson_split64_kernel(const WilsonArg a) {
   const int idx = blockIdx.x * 2 + st;
   const bool ok = idx < n;
   int par = a.out_parity, cb = ok ? idx : n - 1;
-  if (FULLM) full_site(cb, Vh, par, cb);
+  if (FULLM) {
+    par = cb >= Vh;
+    cb -= par * Vh;
+  }
   const char* src = par ? a.in[0] : a.in[1];
   const bool dagger = a.dagger != 0;
   {
