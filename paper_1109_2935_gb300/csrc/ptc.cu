@@ -51,7 +51,7 @@ struct LayerArg {
 struct GradArg {
   InTab x;            // layer inputs [pair][c_in]
   InTab gy;           // dL/dconj(layer output) [pair][c_out]
-  float* partial;     // [pair][p * c_out + c][block][c_in * 32]
+  float* partial;     // [pair][p * A + a][block][N * 32], see WgradShape
   const char* gauge;
   Geom g;
 };
@@ -61,63 +61,86 @@ __device__ __forceinline__ void load_c(const float v[24], C<float> t[12]) {
   for (int k = 0; k < 12; ++k) t[k] = C<float>{v[2 * k], v[2 * k + 1]};
 }
 
-// t = sgn * (U or U^dagger) f on each of the 4 spins
-__device__ __forceinline__ void transport(const Link<float>& U, bool dag, float sgn, const C<float> f[12],
-                                          C<float> t[12]) {
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    C<float> v[3];
-    if (dag) su3_mv_dag(U, f + 3 * s, v);
-    else su3_mv(U, f + 3 * s, v);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) t[3 * s + a] = sgn * v[a];
-  }
-}
-
-// acc[s][a] += sum_t W[s][t] f[t][a]
-__device__ __forceinline__ void spin_mac(C<float> acc[12], const float2* W, const C<float> f[12]) {
+// t = U f (DAG: U^dagger f) on each of the 4 spins. The packed lanes are (re, im) as the
+// fields store them: p = Re(u) f and q = Im(u) f summed over a row, then t = p +- i q.
+template <bool DAG>
+__device__ __forceinline__ void transport(const Link<float>& U, const C<float> f[12], C<float> t[12]) {
 #pragma unroll
   for (int s = 0; s < 4; ++s)
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      float2 w = W[4 * s + t];
-      C<float> wc = {w.x, w.y};
+    for (int a = 0; a < 3; ++a) {
+      float2 p, q;
 #pragma unroll
-      for (int a = 0; a < 3; ++a) cmac(acc[3 * s + a], wc, f[3 * t + a]);
+      for (int b = 0; b < 3; ++b) {
+        const C<float> u = DAG ? U.m[b][a] : U.m[a][b];
+        const float2 h = make_float2(f[3 * s + b].r, f[3 * s + b].i);
+        p = b ? __ffma2_rn(dup2(u.r), h, p) : __fmul2_rn(dup2(u.r), h);
+        q = b ? __ffma2_rn(dup2(u.i), h, q) : __fmul2_rn(dup2(u.i), h);
+      }
+      t[3 * s + a] = DAG ? C<float>{p.x + q.y, p.y - q.x} : C<float>{p.x - q.y, p.y + q.x};
     }
 }
 
-// Neighbour of path p >= 1: its checkerboard index (opposite parity), the link and
-// whether it is applied as U^dagger, and the boundary sign.
+// acc[s][a] += sum_t W[s][t] f[t][a], rows s = 2 sp and 2 sp + 1 of W in the two lanes:
+// W[2 t + sp] = (Re W[2 sp][t], Re W[2 sp + 1][t], Im W[2 sp][t], Im W[2 sp + 1][t]).
+__device__ __forceinline__ void spin_mac(C2 acc[6], const float4* W, const C<float> f[12]) {
+#pragma unroll
+  for (int t = 0; t < 4; ++t)
+#pragma unroll
+    for (int sp = 0; sp < 2; ++sp) {
+      const float4 w = W[2 * t + sp];
+      const float2 wr = make_float2(w.x, w.y), wi = make_float2(w.z, w.w);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const C<float> x = f[3 * t + a];
+        C2& y = acc[3 * sp + a];
+        y.r = __ffma2_rn(wr, dup2(x.r), y.r);
+        y.i = __ffma2_rn(wr, dup2(x.i), y.i);
+        y.r = __ffma2_rn(wi, dup2(-x.i), y.r);
+        y.i = __ffma2_rn(wi, dup2(x.r), y.i);
+      }
+    }
+}
+
+// Neighbour of path p >= 1: its checkerboard index (opposite parity), the link (with the
+// sign of a hop across the antiperiodic t edge) and whether it is applied as U^dagger.
+// p is the same for all threads of a block; the coordinates stay in registers.
 template <int R>
 __device__ __forceinline__ void path_site(const Geom& g, const char* gauge, int p, const int x[4], int par,
-                                          int cb, int& ycb, Link<float>& U, bool& dag, float& sgn) {
+                                          int cb, int& ycb, Link<float>& U, bool& dag) {
   const int mu = (p - 1) >> 1;
   dag = ((p - 1) & 1) != 0;
-  int y[4] = {x[0], x[1], x[2], x[3]};
-  sgn = 1.f;
-  if (!dag) {
-    if (++y[mu] == g.L[mu]) {
-      y[mu] = 0;
-      if (mu == 3 && g.apbc) sgn = -1.f;
+  int y[4];
+  bool edge = false;
+#pragma unroll
+  for (int nu = 0; nu < 4; ++nu) {
+    y[nu] = x[nu];
+    if (nu == mu) {
+      const int last = g.L[nu] - 1;
+      edge = dag ? x[nu] == 0 : x[nu] == last;
+      y[nu] = dag ? (edge ? last : x[nu] - 1) : (edge ? 0 : x[nu] + 1);
     }
-    ycb = cb_index(g, y);
-    LinkIO<P32, R>::load(gauge, g.Vh, mu, par, cb, U);
-  } else {
-    if (y[mu]-- == 0) {
-      y[mu] = g.L[mu] - 1;
-      if (mu == 3 && g.apbc) sgn = -1.f;
-    }
-    ycb = cb_index(g, y);
-    LinkIO<P32, R>::load(gauge, g.Vh, mu, 1 - par, ycb, U);
+  }
+  ycb = cb_index(g, y);
+  LinkIO<P32, R>::load(gauge, g.Vh, mu, dag ? 1 - par : par, dag ? ycb : cb, U);
+  if (mu == 3 && edge && g.apbc) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) U.m[k / 3][k % 3] = C<float>{-U.m[k / 3][k % 3].r, -U.m[k / 3][k % 3].i};
   }
 }
 
+// The layer is bound by the FP32 pipes (36,096 flop per site for channels 1-2-2-1, about
+// 400 bytes): every product rides in packed FP32 instructions, which halve the issue slots;
+// the weights are laid out in shared memory so that one 16-byte read feeds 12 of them.
 template <int CIN, int COUT, int R>
-__global__ void __launch_bounds__(TPB) ptc_layer_kernel(const LayerArg a) {
-  constexpr int NW = NPATH * COUT * CIN * 16;
-  __shared__ float2 sw[NW];
-  for (int i = threadIdx.x; i < NW; i += TPB) sw[i] = a.w[i];
+__global__ void __launch_bounds__(TPB, CIN * COUT <= 4 ? 4 : 1) ptc_layer_kernel(const LayerArg a) {
+  constexpr int NW = NPATH * COUT * CIN * 8;
+  __shared__ float4 sw[NW];
+  for (int i = threadIdx.x; i < NW; i += TPB) {
+    const float2* w = a.w + (i >> 3) * 16 + 8 * (i & 1) + ((i >> 1) & 3);
+    const float2 w0 = w[0], w1 = w[4];
+    sw[i] = make_float4(w0.x, w1.x, w0.y, w1.y);
+  }
   __syncthreads();
   const Geom& g = a.g;
   const int Vh = g.Vh, z = blockIdx.y;
@@ -127,20 +150,19 @@ __global__ void __launch_bounds__(TPB) ptc_layer_kernel(const LayerArg a) {
   const size_t hb = (size_t)96 * Vh;
   int x[4];
   cb_coords(g, cb, par, x);
-  C<float> acc[COUT][12];
+  C2 acc[COUT][6];
 #pragma unroll
   for (int c = 0; c < COUT; ++c)
 #pragma unroll
-    for (int k = 0; k < 12; ++k) acc[c][k] = C<float>{0.f, 0.f};
+    for (int k = 0; k < 6; ++k) acc[c][k] = C2{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 
 #pragma unroll 1
   for (int p = 0; p < NPATH; ++p) {
     int ycb = cb, ypar = par;
     Link<float> U;
     bool dag = false;
-    float sgn = 1.f;
     if (p > 0) {
-      path_site<R>(g, a.gauge, p, x, par, cb, ycb, U, dag, sgn);
+      path_site<R>(g, a.gauge, p, x, par, cb, ycb, U, dag);
       ypar = 1 - par;
     }
     if constexpr (CIN <= COUT) {
@@ -150,19 +172,23 @@ __global__ void __launch_bounds__(TPB) ptc_layer_kernel(const LayerArg a) {
         SpinorIO<P32, 24>::load(a.in.p[z * MAXC + ci] + ypar * hb, Vh, ycb, v);
         C<float> f[12], t[12];
         load_c(v, f);
-        if (p > 0) transport(U, dag, sgn, f, t);
-        else
+        if (p == 0) {
 #pragma unroll
           for (int k = 0; k < 12; ++k) t[k] = f[k];
+        } else if (dag) {
+          transport<true>(U, f, t);
+        } else {
+          transport<false>(U, f, t);
+        }
 #pragma unroll
-        for (int co = 0; co < COUT; ++co) spin_mac(acc[co], sw + ((p * COUT + co) * CIN + ci) * 16, t);
+        for (int co = 0; co < COUT; ++co) spin_mac(acc[co], sw + ((p * COUT + co) * CIN + ci) * 8, t);
       }
     } else {
-      C<float> m[COUT][12];
+      C2 m[COUT][6];
 #pragma unroll
       for (int co = 0; co < COUT; ++co)
 #pragma unroll
-        for (int k = 0; k < 12; ++k) m[co][k] = C<float>{0.f, 0.f};
+        for (int k = 0; k < 6; ++k) m[co][k] = C2{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
       for (int ci = 0; ci < CIN; ++ci) {
         float v[24];
@@ -170,19 +196,23 @@ __global__ void __launch_bounds__(TPB) ptc_layer_kernel(const LayerArg a) {
         C<float> f[12];
         load_c(v, f);
 #pragma unroll
-        for (int co = 0; co < COUT; ++co) spin_mac(m[co], sw + ((p * COUT + co) * CIN + ci) * 16, f);
+        for (int co = 0; co < COUT; ++co) spin_mac(m[co], sw + ((p * COUT + co) * CIN + ci) * 8, f);
       }
 #pragma unroll
       for (int co = 0; co < COUT; ++co) {
         if (p > 0) {
-          C<float> t[12];
-          transport(U, dag, sgn, m[co], t);
+          C2 t[6];
 #pragma unroll
-          for (int k = 0; k < 12; ++k) acc[co][k] = acc[co][k] + t[k];
-        } else {
+          for (int sp = 0; sp < 2; ++sp) {
+            if (dag) su3_mv2<true>(U, m[co] + 3 * sp, t + 3 * sp);
+            else su3_mv2<false>(U, m[co] + 3 * sp, t + 3 * sp);
+          }
 #pragma unroll
-          for (int k = 0; k < 12; ++k) acc[co][k] = acc[co][k] + m[co][k];
+          for (int k = 0; k < 6; ++k) m[co][k] = t[k];
         }
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+          acc[co][k] = C2{__fadd2_rn(acc[co][k].r, m[co][k].r), __fadd2_rn(acc[co][k].i, m[co][k].i)};
       }
     }
   }
@@ -190,95 +220,175 @@ __global__ void __launch_bounds__(TPB) ptc_layer_kernel(const LayerArg a) {
   for (int co = 0; co < COUT; ++co) {
     float v[24];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) { v[2 * k] = acc[co][k].r; v[2 * k + 1] = acc[co][k].i; }
+    for (int sp = 0; sp < 2; ++sp)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const C2 y = acc[co][3 * sp + c];
+        v[12 * sp + 2 * c] = y.r.x; v[12 * sp + 2 * c + 1] = y.i.x;
+        v[12 * sp + 6 + 2 * c] = y.r.y; v[12 * sp + 7 + 2 * c] = y.i.y;
+      }
     SpinorIO<P32, 24>::store(a.out.p[z * MAXC + co] + par * hb, Vh, cb, v);
   }
 }
 
-// blockIdx.y = p * COUT + co, blockIdx.z = pair; grid-stride over the sites.
+// blockIdx.y = p * A + a, blockIdx.z = pair; grid-stride over the sites. The transport of a
+// path is made once per site and block and shared by the N = max(c_in, c_out) contractions:
+// with c_in <= c_out, a block has one input channel a, transports it (t) and contracts it
+// with every g_c; otherwise it has one output channel a and moves the link to the other
+// factor, sum_colour g (U f)^dagger = (U^dagger g) f^dagger. FP32-bound like the layer; one
+// wave of blocks, so that the block sums at the end stay a few percent. Measured on the
+// (2, 2) layer, 16^4 x 4 pairs: 270 us with a transport per (c_in, c_out).
+constexpr int WTPB = 128;  // threads per block
+constexpr int wgrad_ctas(int n) { return n == 1 ? 4 : n == 2 ? 3 : 2; }  // blocks per SM (registers)
+template <int CIN, int COUT>
+struct WgradShape {
+  static constexpr bool FWD = CIN <= COUT;
+  static constexpr int A = FWD ? CIN : COUT, N = FWD ? COUT : CIN;
+};
+
 template <int CIN, int COUT, int R>
-__global__ void __launch_bounds__(GTPB) ptc_wgrad_kernel(const GradArg a) {
-  const int p = blockIdx.y / COUT, co = blockIdx.y % COUT, z = blockIdx.z;
+__global__ void __launch_bounds__(WTPB, (wgrad_ctas(WgradShape<CIN, COUT>::N))) ptc_wgrad_kernel(const GradArg a) {
+  using S = WgradShape<CIN, COUT>;
+  constexpr int N = S::N;
+  const int p = blockIdx.y / S::A, ch = blockIdx.y % S::A, z = blockIdx.z;
   const Geom& g = a.g;
   const int Vh = g.Vh;
   const size_t hb = (size_t)96 * Vh;
-  float acc[CIN][32];
+  // acc[n][sp][t]: rows s = 2 sp, 2 sp + 1 of the 4x4 matrix in the two lanes
+  C2 acc[N][2][4];
 #pragma unroll
-  for (int ci = 0; ci < CIN; ++ci)
+  for (int n = 0; n < N; ++n)
 #pragma unroll
-    for (int k = 0; k < 32; ++k) acc[ci][k] = 0.f;
+    for (int k = 0; k < 8; ++k) acc[n][k >> 2][k & 3] = C2{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 
-  for (int idx = blockIdx.x * GTPB + threadIdx.x; idx < 2 * Vh; idx += gridDim.x * GTPB) {
+  auto load_x = [&](int ci, int par, int cb, C<float> f[12]) {
+    float v[24];
+    SpinorIO<P32, 24>::load(a.x.p[z * MAXC + ci] + par * hb, Vh, cb, v);
+    load_c(v, f);
+  };
+  auto load_g = [&](int co, int par, int cb, C2 gy[6]) {
+    float v[24];
+    SpinorIO<P32, 24>::load(a.gy.p[z * MAXC + co] + par * hb, Vh, cb, v);
+#pragma unroll
+    for (int sp = 0; sp < 2; ++sp)
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        gy[3 * sp + c] = C2{make_float2(v[12 * sp + 2 * c], v[12 * sp + 6 + 2 * c]),
+                            make_float2(v[12 * sp + 2 * c + 1], v[12 * sp + 7 + 2 * c])};
+  };
+  auto contract = [&](C2 q[2][4], const C2 gy[6], const C<float> t[12]) {  // q += gy conj(t)
+#pragma unroll
+    for (int sp = 0; sp < 2; ++sp)
+#pragma unroll
+      for (int tt = 0; tt < 4; ++tt)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const C<float> w = t[3 * tt + c];
+          const C2 y = gy[3 * sp + c];
+          C2& r = q[sp][tt];
+          r.r = __ffma2_rn(dup2(w.r), y.r, r.r);
+          r.i = __ffma2_rn(dup2(w.r), y.i, r.i);
+          r.r = __ffma2_rn(dup2(w.i), y.i, r.r);
+          r.i = __ffma2_rn(dup2(-w.i), y.r, r.i);
+        }
+  };
+
+  for (int idx = blockIdx.x * WTPB + threadIdx.x; idx < 2 * Vh; idx += gridDim.x * WTPB) {
     const int par = idx >= Vh ? 1 : 0, cb = idx - par * Vh;
     int x[4];
     cb_coords(g, cb, par, x);
-    float gv[24];
-    SpinorIO<P32, 24>::load(a.gy.p[z * MAXC + co] + par * hb, Vh, cb, gv);
-    C<float> gy[12];
-    load_c(gv, gy);
     int ycb = cb, ypar = par;
     Link<float> U;
     bool dag = false;
-    float sgn = 1.f;
     if (p > 0) {
-      path_site<R>(g, a.gauge, p, x, par, cb, ycb, U, dag, sgn);
+      path_site<R>(g, a.gauge, p, x, par, cb, ycb, U, dag);
       ypar = 1 - par;
     }
-#pragma unroll
-    for (int ci = 0; ci < CIN; ++ci) {
-      float v[24];
-      SpinorIO<P32, 24>::load(a.x.p[z * MAXC + ci] + ypar * hb, Vh, ycb, v);
+    if constexpr (S::FWD) {
       C<float> f[12], t[12];
-      load_c(v, f);
-      if (p > 0) transport(U, dag, sgn, f, t);
-      else
+      load_x(ch, ypar, ycb, f);
+      if (p == 0) {
 #pragma unroll
         for (int k = 0; k < 12; ++k) t[k] = f[k];
+      } else if (dag) {
+        transport<true>(U, f, t);
+      } else {
+        transport<false>(U, f, t);
+      }
 #pragma unroll
-      for (int s = 0; s < 4; ++s)
+      for (int n = 0; n < N; ++n) {
+        C2 gy[6];
+        load_g(n, par, cb, gy);
+        contract(acc[n], gy, t);
+      }
+    } else {
+      C2 gy[6], w[6];
+      load_g(ch, par, cb, gy);
 #pragma unroll
-        for (int tt = 0; tt < 4; ++tt) {
-          C<float> q = {acc[ci][2 * (4 * s + tt)], acc[ci][2 * (4 * s + tt) + 1]};
+      for (int sp = 0; sp < 2; ++sp) {
+        if (p == 0) {
 #pragma unroll
-          for (int c = 0; c < 3; ++c) cmacc(q, t[3 * tt + c], gy[3 * s + c]);
-          acc[ci][2 * (4 * s + tt)] = q.r;
-          acc[ci][2 * (4 * s + tt) + 1] = q.i;
+          for (int c = 0; c < 3; ++c) w[3 * sp + c] = gy[3 * sp + c];
+        } else if (dag) {
+          su3_mv2<false>(U, gy + 3 * sp, w + 3 * sp);
+        } else {
+          su3_mv2<true>(U, gy + 3 * sp, w + 3 * sp);
         }
+      }
+#pragma unroll
+      for (int n = 0; n < N; ++n) {
+        C<float> f[12];
+        load_x(n, ypar, ycb, f);
+        contract(acc[n], w, f);
+      }
     }
   }
-  constexpr int NV = CIN * 32;
-  __shared__ float red[GTPB / 32][NV];
+  constexpr int NV = N * 32;
+  __shared__ float red[WTPB / 32][NV];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int ci = 0; ci < CIN; ++ci)
+  for (int n = 0; n < N; ++n)
 #pragma unroll
-    for (int k = 0; k < 32; ++k) {
-      float v = acc[ci][k];
+    for (int k = 0; k < 32; ++k) {  // k = 2 (4 s + t) + (0: re, 1: im)
+      const int ss = k >> 3, tt = (k >> 1) & 3;
+      const float2 w = (k & 1) ? acc[n][ss >> 1][tt].i : acc[n][ss >> 1][tt].r;
+      float v = (ss & 1) ? w.y : w.x;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) red[warp][ci * 32 + k] = v;
+      if (lane == 0) red[warp][n * 32 + k] = v;
     }
   __syncthreads();
   float* dst = a.partial + (((size_t)z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * NV;
-  for (int j = threadIdx.x; j < NV; j += GTPB) {
+  for (int j = threadIdx.x; j < NV; j += WTPB) {
     float s = 0.f;
 #pragma unroll
-    for (int w = 0; w < GTPB / 32; ++w) s += red[w][j];
+    for (int w = 0; w < WTPB / 32; ++w) s += red[w][j];
     dst[j] = s;
   }
 }
 
-// grad[(p * COUT + co) * CIN * 32 + ci * 32 + k] = sum over pairs and blocks, FP64, fixed order
-__global__ void ptc_wgrad_reduce(const float* partial, int nblk, int npair, int cout, int cin, double* grad) {
-  const int n = NPATH * cout * cin * 32;
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
-  const int nv = cin * 32, pco = j / nv, r = j % nv;
+// grad[((p * cout + co) * cin + ci) * 32 + k] = sum over pairs and blocks, FP64, fixed order:
+// 32 entries per block, the rows dealt to 8 warps (one thread per entry adding all of them
+// took 19 us).
+constexpr int RROWS = 8;
+__global__ void __launch_bounds__(32 * RROWS)
+    ptc_wgrad_reduce(const float* partial, int nblk, int npair, int cout, int cin, double* grad) {
+  __shared__ double sh[RROWS][32];
+  const bool fwd = cin <= cout;
+  const int na = fwd ? cin : cout, nv = (fwd ? cout : cin) * 32;
+  const int pc = blockIdx.x / cin, ci = blockIdx.x % cin, p = pc / cout, co = pc % cout;
+  const int y = p * na + (fwd ? ci : co), slot = (fwd ? co : ci) * 32 + threadIdx.x;
   double s = 0;
-  for (int z = 0; z < npair; ++z)
-    for (int b = 0; b < nblk; ++b)
-      s += partial[(((size_t)z * NPATH * cout + pco) * nblk + b) * nv + r];
-  grad[j] = s;
+  for (int r = threadIdx.y; r < npair * nblk; r += RROWS) {
+    const int z = r / nblk, b = r - z * nblk;
+    s += partial[(((size_t)z * NPATH * na + y) * nblk + b) * nv + slot];
+  }
+  sh[threadIdx.y][threadIdx.x] = s;
+  __syncthreads();
+  if (threadIdx.y) return;
+#pragma unroll
+  for (int w = 1; w < RROWS; ++w) s += sh[w][threadIdx.x];
+  grad[(size_t)blockIdx.x * 32 + threadIdx.x] = s;
 }
 
 // W'[pbar][ci][co][s][t] = conj(W[p][co][ci][t][s]), pbar the reversed path
@@ -321,13 +431,21 @@ __global__ void __launch_bounds__(GTPB) ptc_norm_kernel(const InTab v, int64_t n
   if (threadIdx.x == 0) partial[(size_t)z * gridDim.x + blockIdx.x] = t;
 }
 
-// inv[z] = 1 / (npair ||v_z||^2) (0 for a zero v)
-__global__ void ptc_inv_kernel(const double* partial, int nblk, int npair, double* inv) {
-  const int z = threadIdx.x;
-  if (z >= npair) return;
+// Sum of n FP64 partial sums by one warp: n / 32 terms per lane, then five shuffles (one
+// thread adding 608 of them took as long as a whole layer).
+__device__ __forceinline__ double warp_total(const double* partial, int n) {
   double s = 0;
-  for (int b = 0; b < nblk; ++b) s += partial[(size_t)z * nblk + b];
-  inv[z] = s > 0 ? 1.0 / (npair * s) : 0.0;
+  for (int b = threadIdx.x; b < n; b += 32) s += partial[b];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// inv[z] = 1 / (npair ||v_z||^2) (0 for a zero v); one warp per pair z = blockIdx.x
+__global__ void ptc_inv_kernel(const double* partial, int nblk, int npair, double* inv) {
+  const int z = blockIdx.x;
+  const double s = warp_total(partial + (size_t)z * nblk, nblk);
+  if (threadIdx.x == 0) inv[z] = s > 0 ? 1.0 / (npair * s) : 0.0;
 }
 
 // d = k - v; gk = inv_z d; partial = inv_z |d|^2 per block
@@ -351,9 +469,8 @@ __global__ void __launch_bounds__(GTPB) ptc_loss_kernel(const InTab k, const InT
 }
 
 __global__ void ptc_sum_kernel(const double* partial, int n, double* out) {
-  double s = 0;
-  for (int i = 0; i < n; ++i) s += partial[i];
-  *out = s;
+  const double s = warp_total(partial, n);
+  if (threadIdx.x == 0) *out = s;
 }
 
 // Adam (Kingma and Ba, Algorithm 1) on theta = (Re W, Im W) with gradient 2 dL/dconj(W);
@@ -392,9 +509,9 @@ void launch_layer(int cin, int cout, int recon, const LayerArg& a, int npair, cu
 
 template <int CIN, int COUT>
 void wgrad_r(int recon, const GradArg& a, dim3 grid, cudaStream_t st) {
-  if (recon == 18) ptc_wgrad_kernel<CIN, COUT, 18><<<grid, GTPB, 0, st>>>(a);
-  else if (recon == 12) ptc_wgrad_kernel<CIN, COUT, 12><<<grid, GTPB, 0, st>>>(a);
-  else ptc_wgrad_kernel<CIN, COUT, 8><<<grid, GTPB, 0, st>>>(a);
+  if (recon == 18) ptc_wgrad_kernel<CIN, COUT, 18><<<grid, WTPB, 0, st>>>(a);
+  else if (recon == 12) ptc_wgrad_kernel<CIN, COUT, 12><<<grid, WTPB, 0, st>>>(a);
+  else ptc_wgrad_kernel<CIN, COUT, 8><<<grid, WTPB, 0, st>>>(a);
 }
 template <int CIN>
 void wgrad_co(int cout, int recon, const GradArg& a, dim3 grid, cudaStream_t st) {
@@ -491,27 +608,26 @@ void run_layer(dirac_ptc* n, int l, const float2* w, int cin, int cout, char* co
   (void)l;
 }
 
-int wgrad(dirac_ptc* n, int l, char* const* x, char* const* gy, int npair, cudaStream_t st) {
-  const int cin = n->ch[l - 1], cout = n->ch[l];
-  const int Vh = n->c->g.Vh;
-  const int maxblk = (2 * Vh + GTPB - 1) / GTPB;
-  int nblk = (152 * 8 + NPATH * cout * npair - 1) / (NPATH * cout * npair);
-  nblk = std::max(1, std::min(nblk, maxblk));
-  size_t need = (size_t)npair * NPATH * cout * nblk * cin * 32 * sizeof(float);
-  int rc = grow(n, reinterpret_cast<char**>(&n->partial), &n->partial_bytes, need);
+int wgrad(dirac_ptc* net, int l, char* const* x, char* const* gy, int npair, cudaStream_t st) {
+  const int cin = net->ch[l - 1], cout = net->ch[l];
+  const int Vh = net->c->g.Vh;
+  const int na = std::min(cin, cout), n = std::max(cin, cout);
+  const int maxblk = (2 * Vh + WTPB - 1) / WTPB;
+  const int nblk = std::max(1, std::min(152 * wgrad_ctas(n) / (NPATH * na * npair), maxblk));
+  size_t need = (size_t)npair * NPATH * na * nblk * n * 32 * sizeof(float);
+  int rc = grow(net, reinterpret_cast<char**>(&net->partial), &net->partial_bytes, need);
   if (rc) return rc;
   GradArg a{};
   for (int z = 0; z < npair; ++z) {
     for (int c = 0; c < cin; ++c) a.x.p[z * MAXC + c] = x[z * MAXC + c];
     for (int c = 0; c < cout; ++c) a.gy.p[z * MAXC + c] = gy[z * MAXC + c];
   }
-  a.partial = n->partial;
-  a.gauge = n->c->gauge[P32];
-  a.g = geom(n);
-  launch_wgrad(cin, cout, n->c->p.recon[P32], a, dim3(nblk, NPATH * cout, npair), st);
-  const int nv = NPATH * cout * cin * 32;
-  ptc_wgrad_reduce<<<(nv + 127) / 128, 128, 0, st>>>(n->partial, nblk, npair, cout, cin,
-                                                     n->grad + 2 * n->woff[l - 1]);
+  a.partial = net->partial;
+  a.gauge = net->c->gauge[P32];
+  a.g = geom(net);
+  launch_wgrad(cin, cout, net->c->p.recon[P32], a, dim3(nblk, NPATH * na, npair), st);
+  ptc_wgrad_reduce<<<NPATH * cout * cin, dim3(32, RROWS), 0, st>>>(net->partial, nblk, npair, cout, cin,
+                                                                 net->grad + 2 * net->woff[l - 1]);
   return DIRAC_OK;
 }
 
@@ -567,9 +683,9 @@ int forward_backward(dirac_ptc* n, const Work& W, const char* const* r, const ch
   }
   double* part = n->dsc + DSC_PARTIAL;
   ptc_norm_kernel<<<dim3(NORM_BLOCKS, B), GTPB, 0, st>>>(vt, n4, part);
-  ptc_inv_kernel<<<1, 32, 0, st>>>(part, NORM_BLOCKS, B, n->dsc);
+  ptc_inv_kernel<<<B, 32, 0, st>>>(part, NORM_BLOCKS, B, n->dsc);
   ptc_loss_kernel<<<dim3(NORM_BLOCKS, B), GTPB, 0, st>>>(kt, vt, gt, n->dsc, n4, part);
-  ptc_sum_kernel<<<1, 1, 0, st>>>(part, NORM_BLOCKS * B, n->dsc + MAXB);
+  ptc_sum_kernel<<<1, 32, 0, st>>>(part, NORM_BLOCKS * B, n->dsc + MAXB);
   if (!grads) return DIRAC_OK;
   for (int l = L; l >= 1; --l) {
     std::vector<char*> x(MAXB * MAXC), gy(MAXB * MAXC), gx(MAXB * MAXC);
