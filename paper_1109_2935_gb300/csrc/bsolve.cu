@@ -75,6 +75,51 @@ __device__ __forceinline__ void store_v(const Seg& g, int v, int r, int s, const
   SpinorIO<PREC, 24>::store(b, g.Vh, cb, t);
 }
 
+// store_v, leaving in `in` the values as stored (what a reload would give, without it)
+template <int PREC, typename T>
+__device__ __forceinline__ void store_q(const Seg& g, int v, int r, int s, T in[24]) {
+  if constexpr (PREC == P16) {
+    int cb;
+    char* b = const_cast<char*>(site_base(g, v, r, s, cb));
+    float inv;
+    const float n = site_norm_scale(in, 24, inv);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      float w[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) w[j] = in[8 * k + j] * inv;
+      const int4 q = pack_half8(w);
+      *reinterpret_cast<int4*>(b + ((size_t)k * g.Vh + cb) * 16) = q;
+      unpack_half8(q, w);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) in[8 * k + j] = w[j] * n;
+    }
+    reinterpret_cast<float*>(b + (size_t)48 * g.Vh)[cb] = n;
+  } else {
+    store_v<PREC>(g, v, r, s, in);
+  }
+}
+
+// a site of an FP16 vector as stored; chunk(c) decodes 8 of its reals as a load does
+struct RawS {
+  int4 q[3];
+  float n;
+  __device__ __forceinline__ void chunk(int c, float v[8]) const {
+    unpack_half8(q[c], v);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] *= n;
+  }
+};
+__device__ __forceinline__ RawS raw_s(const Seg& g, int v, int r, int s) {
+  int cb;
+  const char* b = site_base(g, v, r, s, cb);
+  RawS t;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) t.q[k] = *reinterpret_cast<const int4*>(b + ((size_t)k * g.Vh + cb) * 16);
+  t.n = reinterpret_cast<const float*>(b + (size_t)48 * g.Vh)[cb];
+  return t;
+}
+
 // ---------------------------------------------------------------- operations
 // op(g, r, s, sc, acc): site s of local right-hand side r; sc = its scalar state
 template <int SP> struct OpPUpd {  // p = rs + beta p + nbw v
@@ -155,6 +200,46 @@ template <int SP, int AP> struct OpXR {
     const T ar = (T)sc[SC_ALPHA], ai = (T)sc[SC_ALPHA + 1];
     const T wr = (T)sc[SC_OMEGA], wi = (T)sc[SC_OMEGA + 1];
     const T nr = (T)sc[SC_NOMEGA], ni = (T)sc[SC_NOMEGA + 1];
+    if constexpr (SP == P16 && AP == P32) {
+      // every input in its stored form first (76 registers), decoded chunk by chunk
+      const RawS rp = raw_s(g, VP, r, s), ru = raw_s(g, VRS, r, s), rt = raw_s(g, VT, r, s), rz = raw_s(g, VR0, r, s);
+      float x[24], u[24];
+      load_v<P32>(g, VXS, r, s, x);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        float p[8], t[8], w[8];
+        rp.chunk(c, p);
+        ru.chunk(c, w);
+        rt.chunk(c, t);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int k = 4 * c + j;
+          x[2 * k] += ar * p[2 * j] - ai * p[2 * j + 1] + wr * w[2 * j] - wi * w[2 * j + 1];
+          x[2 * k + 1] += ar * p[2 * j + 1] + ai * p[2 * j] + wr * w[2 * j + 1] + wi * w[2 * j];
+          u[2 * k] = w[2 * j] + (nr * t[2 * j] - ni * t[2 * j + 1]);
+          u[2 * k + 1] = w[2 * j + 1] + (nr * t[2 * j + 1] + ni * t[2 * j]);
+        }
+      }
+      store_v<P32>(g, VXS, r, s, x);
+      store_q<P16>(g, VRS, r, s, u);
+      float rr = 0, re = 0, im = 0;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        float z[8];
+        rz.chunk(c, z);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float ur = u[8 * c + 2 * j], ui = u[8 * c + 2 * j + 1];
+          rr += ur * ur + ui * ui;
+          re += z[2 * j] * ur + z[2 * j + 1] * ui;
+          im += z[2 * j] * ui - z[2 * j + 1] * ur;
+        }
+      }
+      acc[0] += rr;
+      acc[1] += re;
+      acc[2] += im;
+      return;
+    }
     T p[24], u[24], t[24], x[24], z[24];
     load_v<SP>(g, VP, r, s, p);
     load_v<SP>(g, VRS, r, s, u);
@@ -169,8 +254,7 @@ template <int SP, int AP> struct OpXR {
       u[2 * k + 1] += nr * t[2 * k + 1] + ni * t[2 * k];
     }
     store_v<AP>(g, VXS, r, s, x);
-    store_v<SP>(g, VRS, r, s, u);
-    load_v<SP>(g, VRS, r, s, u);  // the residual as stored
+    store_q<SP>(g, VRS, r, s, u);  // the residual as stored
     T rr = 0, re = 0, im = 0;
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
@@ -301,8 +385,14 @@ __device__ __forceinline__ void block_sum(const double* acc, RedShared<NRED>& sh
 // (deterministic) into its scalar slots.
 // A right-hand side whose mask entry (mask[rhs * mstride], when mask is given) is 0 is
 // skipped by all its blocks: no site work, no partial sums, its ticket untouched.
+// CTAs per SM: the update of x and r holds five vectors of a site; capped to two CTAs (128
+// registers instead of 178 and one CTA) it has twice the loads in flight.
+template <class Op> struct MinCtas { static constexpr int n = 1; };
+template <int AP> struct MinCtas<OpXR<P16, AP>> { static constexpr int n = 2; };
+template <> struct MinCtas<OpPUpd<P16>> { static constexpr int n = 3; };
+
 template <class Op>
-__global__ void __launch_bounds__(NT) mb_kernel(const Seg* __restrict__ segs, int nseg, Op op, double* scal,
+__global__ void __launch_bounds__(NT, MinCtas<Op>::n) mb_kernel(const Seg* __restrict__ segs, int nseg, Op op, double* scal,
                                                 double* part, unsigned* tick, const double* mask, int mstride) {
   int l = 0;
   while (l + 1 < nseg && (int)blockIdx.x >= segs[l + 1].blk0) ++l;
