@@ -136,88 +136,119 @@ __device__ __forceinline__ void load_link_h(const char* base, int Vh, int mu, in
   }
 }
 
-template <int PREC, int RL>
+// One hop: acc += f r, with r the link product of the neighbour n mu (n = +-1: fat link,
+// +-3: long link) and f its phase, boundary sign and (16-bit storage) norm.
+template <int PREC, int RL, bool LONG, bool BACK, typename T>
+__device__ __forceinline__ void stag_hop(const StagArg& a, const int x[4], int cb, int mu, T eta, C<T> r[3], T& f) {
+  const Geom& g = a.g;
+  const int Vh = g.Vh, par = a.out_parity;
+  constexpr int n = (BACK ? -1 : 1) * (LONG ? 3 : 1);
+  const char* links = LONG ? a.lng : a.fat;
+  int v = 0, L = 1, stride = 1;  // selects: mu may differ from lane to lane
+#pragma unroll
+  for (int nu = 0, s = g.Lxh; nu < 4; ++nu) {
+    if (nu == mu) {
+      v = x[nu];
+      L = g.L[nu];
+      stride = s;
+    }
+    if (nu > 0) s *= g.L[nu];
+  }
+  int w;
+  const int y = stag_shift(v, n, L, w);
+  const int ycb = mu == 0 ? cb + (y >> 1) - (v >> 1) : cb + (y - v) * stride;
+  const T bc = (mu == 3 && g.apbc && (w & 1)) ? (T)-1 : (T)1;
+  // forward: link at x; backward: link (adjoint) at the neighbour
+  const int lpar = BACK ? 1 - par : par, lcb = BACK ? ycb : cb;
+  constexpr int RR = LONG ? RL : 18;
+  T nrm;
+  if constexpr (PREC == P16 && RL != 8) {
+    uint32_t chi[3], uw[9];
+    nrm = load_stag_h(a.in, Vh, ycb, chi);
+    load_link_h<RR>(links, Vh, mu, lpar, lcb, uw);
+    stag_mv_h<RR>(uw, chi, BACK, r);
+  } else {
+    T q[6];
+    nrm = load_stag_spinor<PREC, T>(a.in, Vh, ycb, q);
+    const C<T> h[3] = {{q[0], q[1]}, {q[2], q[3]}, {q[4], q[5]}};
+    Link<T> U;
+    LinkIO<PREC, RR>::load(links, Vh, mu, lpar, lcb, U);
+    if (BACK) su3_mv_dag(U, h, r);
+    else su3_mv(U, h, r);
+  }
+  f = (BACK ? -eta : eta) * bc * nrm;
+}
+
+// LANES = 1: a thread per output site. LANES = 4: the four directions of a site on four
+// neighbouring lanes; the sum passes from lane to lane in the order of LANES = 1, so the
+// results are the same bits. A small lattice is bound by the latency of a thread's 16 hops
+// (2 to 3 of them in flight), which four lanes share.
+template <int PREC, int RL, int LANES>
 __global__ void __launch_bounds__(128) staggered_kernel(const StagArg a) {
   using T = typename Real<PREC>::T;
   const Geom& g = a.g;
   const int Vh = g.Vh;
-  int cb = blockIdx.x * blockDim.x + threadIdx.x;
-  if (cb >= Vh) return;
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = LANES == 1 ? 0 : threadIdx.x % LANES;
+  int cb = LANES == 1 ? idx : idx / LANES;
+  const bool ok = cb < Vh;
+  if (LANES == 1 && !ok) return;
+  if (!ok) cb = Vh - 1;  // lanes past the end keep their warp's exchange whole
   const int par = a.out_parity;
   int x[4];
   cb_coords(g, cb, par, x);
   C<T> acc[3] = {{0, 0}, {0, 0}, {0, 0}};
-  int esum = 0;
+  if constexpr (LANES == 1) {
+    int esum = 0;
 #pragma unroll
-  for (int mu = 0; mu < 4; ++mu) {
+    for (int mu = 0; mu < 4; ++mu) {
+      const T eta = (esum & 1) ? (T)-1 : (T)1;
+      esum += x[mu];
+      C<T> r[3];
+      T f;
+      auto add = [&] {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) acc[c] = C<T>{fma(f, r[c].r, acc[c].r), fma(f, r[c].i, acc[c].i)};
+      };
+      stag_hop<PREC, RL, false, false, T>(a, x, cb, mu, eta, r, f);
+      add();
+      stag_hop<PREC, RL, false, true, T>(a, x, cb, mu, eta, r, f);
+      add();
+      stag_hop<PREC, RL, true, false, T>(a, x, cb, mu, eta, r, f);
+      add();
+      stag_hop<PREC, RL, true, true, T>(a, x, cb, mu, eta, r, f);
+      add();
+    }
+  } else {
+    int esum = 0;
+#pragma unroll
+    for (int nu = 0; nu < 3; ++nu) esum += nu < lane ? x[nu] : 0;
     const T eta = (esum & 1) ? (T)-1 : (T)1;
-    esum += x[mu];
+    C<T> r[4][3];
+    T f[4];
+    stag_hop<PREC, RL, false, false, T>(a, x, cb, lane, eta, r[0], f[0]);
+    stag_hop<PREC, RL, false, true, T>(a, x, cb, lane, eta, r[1], f[1]);
+    stag_hop<PREC, RL, true, false, T>(a, x, cb, lane, eta, r[2], f[2]);
+    stag_hop<PREC, RL, true, true, T>(a, x, cb, lane, eta, r[3], f[3]);
 #pragma unroll
-    for (int hop = 0; hop < 2; ++hop) {
-      const int n = hop == 0 ? 1 : 3;
-      const char* links = hop == 0 ? a.fat : a.lng;
-      // forward: link at x, neighbour x + n mu
-      {
-        int y[4] = {x[0], x[1], x[2], x[3]}, w;
-        y[mu] = stag_shift(x[mu], n, g.L[mu], w);
-        T bc = (mu == 3 && g.apbc && (w & 1)) ? (T)-1 : (T)1;
-        C<T> r[3];
-        T nrm;
-        if constexpr (PREC == P16 && RL != 8) {
-          uint32_t chi[3], uw[9];
-          nrm = load_stag_h(a.in, Vh, cb_index(g, y), chi);
-          if (hop == 0) {
-            load_link_h<18>(links, Vh, mu, par, cb, uw);
-            stag_mv_h<18>(uw, chi, false, r);
-          } else {
-            load_link_h<RL>(links, Vh, mu, par, cb, uw);
-            stag_mv_h<RL>(uw, chi, false, r);
-          }
-        } else {
-          T v[6];
-          nrm = load_stag_spinor<PREC, T>(a.in, Vh, cb_index(g, y), v);
-          C<T> h[3] = {{v[0], v[1]}, {v[2], v[3]}, {v[4], v[5]}};
-          Link<T> U;
-          if (hop == 0) LinkIO<PREC, 18>::load(links, Vh, mu, par, cb, U);
-          else LinkIO<PREC, RL>::load(links, Vh, mu, par, cb, U);
-          su3_mv(U, h, r);
-        }
-        const T f = eta * bc * nrm;
+    for (int m = 0; m < 4; ++m) {
+      if (lane == m) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) acc[c] = acc[c] + f * r[c];
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+          for (int c = 0; c < 3; ++c)
+            acc[c] = C<T>{fma(f[k], r[k][c].r, acc[c].r), fma(f[k], r[k][c].i, acc[c].i)};
       }
-      // backward: link at x - n mu, neighbour x - n mu
-      {
-        int y[4] = {x[0], x[1], x[2], x[3]}, w;
-        y[mu] = stag_shift(x[mu], -n, g.L[mu], w);
-        T bc = (mu == 3 && g.apbc && (w & 1)) ? (T)-1 : (T)1;
-        int ycb = cb_index(g, y);
-        C<T> r[3];
-        T nrm;
-        if constexpr (PREC == P16 && RL != 8) {
-          uint32_t chi[3], uw[9];
-          nrm = load_stag_h(a.in, Vh, ycb, chi);
-          if (hop == 0) {
-            load_link_h<18>(links, Vh, mu, 1 - par, ycb, uw);
-            stag_mv_h<18>(uw, chi, true, r);
-          } else {
-            load_link_h<RL>(links, Vh, mu, 1 - par, ycb, uw);
-            stag_mv_h<RL>(uw, chi, true, r);
-          }
-        } else {
-          T v[6];
-          nrm = load_stag_spinor<PREC, T>(a.in, Vh, ycb, v);
-          C<T> h[3] = {{v[0], v[1]}, {v[2], v[3]}, {v[4], v[5]}};
-          Link<T> U;
-          if (hop == 0) LinkIO<PREC, 18>::load(links, Vh, mu, 1 - par, ycb, U);
-          else LinkIO<PREC, RL>::load(links, Vh, mu, 1 - par, ycb, U);
-          su3_mv_dag(U, h, r);
-        }
-        const T f = -eta * bc * nrm;
+      if (m < 3) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) acc[c] = acc[c] + f * r[c];
+        for (int c = 0; c < 3; ++c) {
+          const T pr = __shfl_up_sync(0xffffffffu, acc[c].r, 1, LANES);
+          const T pi = __shfl_up_sync(0xffffffffu, acc[c].i, 1, LANES);
+          if (lane == m + 1) acc[c] = C<T>{pr, pi};
+        }
       }
     }
+    if (lane != LANES - 1 || !ok) return;
   }
   T out[6];
   const T bb = (T)a.b;
@@ -236,12 +267,24 @@ __global__ void __launch_bounds__(128) staggered_kernel(const StagArg a) {
   SpinorIO<PREC, 6>::store(a.out, Vh, cb, out);
 }
 
+template <int PREC, int LANES>
+static void launch_stag_lanes(int recon, const StagArg& a, cudaStream_t st) {
+  const int per = 128 / LANES;
+  dim3 block(128), grid((a.g.Vh + per - 1) / per);
+  if (recon == 18) staggered_kernel<PREC, 18, LANES><<<grid, block, 0, st>>>(a);
+  else if (recon == 12) staggered_kernel<PREC, 12, LANES><<<grid, block, 0, st>>>(a);
+  else staggered_kernel<PREC, 8, LANES><<<grid, block, 0, st>>>(a);
+}
+
+// Up to this many output sites four lanes share a site. Measured (two launches, us, one lane
+// -> four): FP32 4,096 sites 16.6 -> 9.7, 13,824 16.6 -> 12.5, 32,768 16.6 -> 20.7; FP16
+// 13,824 16.6 -> 12.5, 32,768 16.6 -> 16.5; FP64 4,096 57.6 -> 24.8, 13,824 59.7 -> 61.6.
+template <int PREC> constexpr int kStagSplitSites = PREC == P64 ? 8192 : 16384;
+
 template <int PREC>
 static void launch_stag_prec(int recon, const StagArg& a, cudaStream_t st) {
-  dim3 block(128), grid((a.g.Vh + 127) / 128);
-  if (recon == 18) staggered_kernel<PREC, 18><<<grid, block, 0, st>>>(a);
-  else if (recon == 12) staggered_kernel<PREC, 12><<<grid, block, 0, st>>>(a);
-  else staggered_kernel<PREC, 8><<<grid, block, 0, st>>>(a);
+  if (a.g.Vh <= kStagSplitSites<PREC>) launch_stag_lanes<PREC, 4>(recon, a, st);
+  else launch_stag_lanes<PREC, 1>(recon, a, st);
 }
 
 void launch_staggered(int prec, int recon, char* out, const char* in, const char* x,
