@@ -638,6 +638,7 @@ template <class Op> struct MinBlocks<Op, std::void_t<decltype(Op::kMinBlocks)>> 
 
 template <class Op>
 __global__ void __launch_bounds__(kThreads, MinBlocks<Op>::value) blas_map_kernel(Op op, int n) {
+  pdl_begin();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) op(i, nullptr);
 }
 
@@ -674,6 +675,7 @@ __device__ __forceinline__ void block_sum3(const double acc[3], RedShared& sh) {
 template <class Op>
 __global__ void __launch_bounds__(kThreads, MinBlocks<Op>::value) blas_reduce_kernel(Op op, int n, double* partials,
                                                           unsigned* ticket, double* res) {
+  pdl_begin();
   __shared__ RedShared sh;
   double acc[3] = {0, 0, 0};
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) op(i, acc);
@@ -714,7 +716,7 @@ static int run_map(Blas* b, const Op& op, int n, cudaStream_t st) {
   int grid = (n + kThreads - 1) / kThreads;
   if (grid > kMaxGrid) grid = kMaxGrid;
   if (grid < 1) grid = 1;
-  blas_map_kernel<Op><<<grid, kThreads, 0, st>>>(op, n);
+  launch_pdl(blas_map_kernel<Op>, grid, kThreads, 0, st, op, n);
   return check(b, "blas map kernel");
 }
 
@@ -727,7 +729,7 @@ static int run_reduce(Blas* b, const Op& op, int n, double* out, int nout, cudaS
   int grid = (n + kThreads - 1) / kThreads;
   if (grid > kMaxGrid) grid = kMaxGrid;
   if (grid < 1) grid = 1;
-  blas_reduce_kernel<Op><<<grid, kThreads, 0, st>>>(op, n, b->partials, b->ticket, dres ? dres : b->dev_res);
+  launch_pdl(blas_reduce_kernel<Op>, grid, kThreads, 0, st, op, n, b->partials, b->ticket, dres ? dres : b->dev_res);
   int rc = check(b, "blas reduce kernel");
   if (rc || dres) return rc;  // device-resident result: no synchronisation
   cudaError_t e = cudaStreamSynchronize(st);

@@ -394,6 +394,7 @@ template <> struct MinCtas<OpPUpd<P16>> { static constexpr int n = 3; };
 template <class Op>
 __global__ void __launch_bounds__(NT, MinCtas<Op>::n) mb_kernel(const Seg* __restrict__ segs, int nseg, Op op, double* scal,
                                                 double* part, unsigned* tick, const double* mask, int mstride) {
+  pdl_begin();
   int l = 0;
   while (l + 1 < nseg && (int)blockIdx.x >= segs[l + 1].blk0) ++l;
   const Seg& g = segs[l];
@@ -440,6 +441,7 @@ __device__ __forceinline__ void fail(double* S, int f) {
 }
 // beta = (rho / rho_old)(alpha / omega); nbw = -beta omega
 __global__ void k_b1(double* scal, int n) {
+  pdl_begin();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
   double* S = scal + (size_t)j * NSC;
@@ -463,6 +465,7 @@ __global__ void k_b1(double* scal, int n) {
 }
 // alpha = rho / (r0, v)
 __global__ void k_b2(double* scal, int n) {
+  pdl_begin();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
   double* S = scal + (size_t)j * NSC;
@@ -478,6 +481,7 @@ __global__ void k_b2(double* scal, int n) {
 }
 // omega = (t, s) / (t, t)
 __global__ void k_b3(double* scal, int n) {
+  pdl_begin();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
   double* S = scal + (size_t)j * NSC;
@@ -498,6 +502,7 @@ __global__ void k_b3(double* scal, int n) {
 }
 // rho_old = rho; rho = (r0, r); mirror ||r||^2 and the flag for the host
 __global__ void k_b4(double* scal, int n, double* mirror) {
+  pdl_begin();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
   double* S = scal + (size_t)j * NSC;
@@ -512,6 +517,7 @@ __global__ void k_b4(double* scal, int n, double* mirror) {
 // start / after a reliable update of the right-hand sides with upd[j] != 0: rho = (r0, rs)
 // (in SC_TMP); active flags from the host
 __global__ void k_restart(double* scal, int n, const double* active, const double* upd, int first) {
+  pdl_begin();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n || upd[j] == 0.0) return;
   double* S = scal + (size_t)j * NSC;
@@ -526,6 +532,7 @@ __global__ void k_restart(double* scal, int n, const double* active, const doubl
 }
 // per-right-hand-side value of a scalar slot into host-visible memory
 __global__ void k_gather(const double* scal, int n, int slot, double* out) {
+  pdl_begin();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j < n) out[j] = scal[(size_t)j * NSC + slot];
 }
@@ -590,16 +597,16 @@ template <class Op>
 int launch(Run& R, const Op& op, int which = ALL) {
   const double* mask = which == ACTIVE ? R.scal + SC_ACTIVE : (which == UPDATING ? R.upd_d() : nullptr);
   const int stride = which == ACTIVE ? NSC : 1;
-  mb_kernel<Op><<<R.nblk, NT, 0, R.st>>>(R.d_segs, R.nseg, op, R.scal, R.part, R.tick, mask, stride);
+  launch_pdl(mb_kernel<Op>, R.nblk, NT, 0, R.st, R.d_segs, R.nseg, op, R.scal, R.part, R.tick, mask, stride);
   return cudaGetLastError() == cudaSuccess ? DIRAC_OK : DIRAC_ERR_CUDA;
 }
 int scalar(Run& R, int which, int slot = 0) {
   const int g = (R.nrhs + 63) / 64;
   switch (which) {
-    case 1: k_b1<<<g, 64, 0, R.st>>>(R.scal, R.nrhs); break;
-    case 2: k_b2<<<g, 64, 0, R.st>>>(R.scal, R.nrhs); break;
-    case 3: k_b3<<<g, 64, 0, R.st>>>(R.scal, R.nrhs); break;
-    case 4: k_b4<<<g, 64, 0, R.st>>>(R.scal, R.nrhs, R.mirror(slot)); break;
+    case 1: launch_pdl(k_b1, g, 64, 0, R.st, R.scal, R.nrhs); break;
+    case 2: launch_pdl(k_b2, g, 64, 0, R.st, R.scal, R.nrhs); break;
+    case 3: launch_pdl(k_b3, g, 64, 0, R.st, R.scal, R.nrhs); break;
+    case 4: launch_pdl(k_b4, g, 64, 0, R.st, R.scal, R.nrhs, R.mirror(slot)); break;
   }
   return cudaGetLastError() == cudaSuccess ? DIRAC_OK : DIRAC_ERR_CUDA;
 }
@@ -634,7 +641,7 @@ int iteration(Run& R, int slot) {
 int residual(Run& R, dirac_batch* plan) {
   RT(dirac_batch_apply(plan, R.st));   // r = M x
   RT(launch(R, OpXmy{}, UPDATING));
-  k_gather<<<(R.nrhs + 63) / 64, 64, 0, R.st>>>(R.scal, R.nrhs, SC_RR, R.gathered());
+  launch_pdl(k_gather, (R.nrhs + 63) / 64, 64, 0, R.st, R.scal, R.nrhs, SC_RR, R.gathered());
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(R.st) != cudaSuccess) return DIRAC_ERR_CUDA;
   return DIRAC_OK;
 }
@@ -650,7 +657,7 @@ int restart(Run& R, int first) {
   RT(launch(R, OpRestart<SP, AP>{}, UPDATING));
   RT(launch(R, OpCdot<SP, VR0, VRS, SC_TMP>{}, UPDATING));
   // the host's active flags (pinned, mapped) for the scalar state
-  k_restart<<<(R.nrhs + 63) / 64, 64, 0, R.st>>>(R.scal, R.nrhs, R.active_d(), R.upd_d(), first);
+  launch_pdl(k_restart, (R.nrhs + 63) / 64, 64, 0, R.st, R.scal, R.nrhs, R.active_d(), R.upd_d(), first);
   return cudaGetLastError() == cudaSuccess ? DIRAC_OK : DIRAC_ERR_CUDA;
 }
 
@@ -661,7 +668,7 @@ int solve_batched_impl(Run& R, const dirac_solver_params& P, dirac_solver_stats*
   const int n = R.nrhs;
   // ||b||^2, r = b, x = 0 (or r = b - M x from the initial guess)
   RT(launch(R, OpNormB{}));
-  k_gather<<<(n + 63) / 64, 64, 0, R.st>>>(R.scal, n, SC_BB, R.gathered());
+  launch_pdl(k_gather, (n + 63) / 64, 64, 0, R.st, R.scal, n, SC_BB, R.gathered());
   if (cudaStreamSynchronize(R.st) != cudaSuccess) return DIRAC_ERR_CUDA;
   std::vector<double> target(n), rmax(n), rr(n);
   std::vector<int> active(n, 1), relup(n, 0), stale(n, 0);
@@ -681,7 +688,7 @@ int solve_batched_impl(Run& R, const dirac_solver_params& P, dirac_solver_stats*
     RT(launch(R, OpXmy{}));
     RT(launch(R, OpRestart<SP, AP>{}));
     RT(launch(R, OpShadow<SP>{}));
-    k_gather<<<(n + 63) / 64, 64, 0, R.st>>>(R.scal, n, SC_RR, R.gathered());
+    launch_pdl(k_gather, (n + 63) / 64, 64, 0, R.st, R.scal, n, SC_RR, R.gathered());
     if (cudaStreamSynchronize(R.st) != cudaSuccess) return DIRAC_ERR_CUDA;
     for (int j = 0; j < n; ++j) rr[j] = R.hgathered()[j];
   } else {

@@ -10,7 +10,34 @@
 #include <cstdint>
 #include <type_traits>
 
+#include <utility>
+
 namespace dirac {
+
+// Launches that follow one another on a stream (the steps of a solver, the hops of an
+// even-odd operator) start without the gap between two kernels: launch_pdl lets a grid
+// become resident while its predecessor runs, and pdl_begin, the first statement of every
+// kernel launched this way, waits until that predecessor is complete and its writes are
+// visible, then lets the successor come up. Without the attribute both are no-ops, and any
+// other work on the stream is ordered as ever.
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);
+}
 
 enum { P64 = 0, P32 = 1, P16 = 2 };
 // a fourth arithmetic for stencils only: FP64 storage read into double-single (float-float)

@@ -134,6 +134,7 @@ __device__ __forceinline__ void path_site(const Geom& g, const char* gauge, int 
 // the weights are laid out in shared memory so that one 16-byte read feeds 12 of them.
 template <int CIN, int COUT, int R>
 __global__ void __launch_bounds__(TPB, CIN * COUT <= 4 ? 4 : 1) ptc_layer_kernel(const LayerArg a) {
+  pdl_begin();
   constexpr int NW = NPATH * COUT * CIN * 8;
   __shared__ float4 sw[NW];
   for (int i = threadIdx.x; i < NW; i += TPB) {
@@ -248,6 +249,7 @@ struct WgradShape {
 
 template <int CIN, int COUT, int R>
 __global__ void __launch_bounds__(WTPB, (wgrad_ctas(WgradShape<CIN, COUT>::N))) ptc_wgrad_kernel(const GradArg a) {
+  pdl_begin();
   using S = WgradShape<CIN, COUT>;
   constexpr int N = S::N;
   const int p = blockIdx.y / S::A, ch = blockIdx.y % S::A, z = blockIdx.z;
@@ -373,6 +375,7 @@ __global__ void __launch_bounds__(WTPB, (wgrad_ctas(WgradShape<CIN, COUT>::N))) 
 constexpr int RROWS = 8;
 __global__ void __launch_bounds__(32 * RROWS)
     ptc_wgrad_reduce(const float* partial, int nblk, int npair, int cout, int cin, double* grad) {
+  pdl_begin();
   __shared__ double sh[RROWS][32];
   const bool fwd = cin <= cout;
   const int na = fwd ? cin : cout, nv = (fwd ? cout : cin) * 32;
@@ -393,6 +396,7 @@ __global__ void __launch_bounds__(32 * RROWS)
 
 // W'[pbar][ci][co][s][t] = conj(W[p][co][ci][t][s]), pbar the reversed path
 __global__ void ptc_adjoint_kernel(const float2* w, float2* wa, int cout, int cin) {
+  pdl_begin();
   const int n = NPATH * cout * cin * 16;
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
@@ -419,6 +423,7 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 
 // partial[z * gridDim.x + block] = sum |v_z|^2 over the block's float4 chunks
 __global__ void __launch_bounds__(GTPB) ptc_norm_kernel(const InTab v, int64_t n4, double* partial) {
+  pdl_begin();
   __shared__ double sh[GTPB / 32];
   const int z = blockIdx.y;
   const float4* p = reinterpret_cast<const float4*>(v.p[z * MAXC]);
@@ -443,6 +448,7 @@ __device__ __forceinline__ double warp_total(const double* partial, int n) {
 
 // inv[z] = 1 / (npair ||v_z||^2) (0 for a zero v); one warp per pair z = blockIdx.x
 __global__ void ptc_inv_kernel(const double* partial, int nblk, int npair, double* inv) {
+  pdl_begin();
   const int z = blockIdx.x;
   const double s = warp_total(partial + (size_t)z * nblk, nblk);
   if (threadIdx.x == 0) inv[z] = s > 0 ? 1.0 / (npair * s) : 0.0;
@@ -451,6 +457,7 @@ __global__ void ptc_inv_kernel(const double* partial, int nblk, int npair, doubl
 // d = k - v; gk = inv_z d; partial = inv_z |d|^2 per block
 __global__ void __launch_bounds__(GTPB) ptc_loss_kernel(const InTab k, const InTab v, OutTab gk, const double* inv,
                                                         int64_t n4, double* partial) {
+  pdl_begin();
   __shared__ double sh[GTPB / 32];
   const int z = blockIdx.y;
   const float4* kp = reinterpret_cast<const float4*>(k.p[z * MAXC]);
@@ -469,6 +476,7 @@ __global__ void __launch_bounds__(GTPB) ptc_loss_kernel(const InTab k, const InT
 }
 
 __global__ void ptc_sum_kernel(const double* partial, int n, double* out) {
+  pdl_begin();
   const double s = warp_total(partial, n);
   if (threadIdx.x == 0) *out = s;
 }
@@ -477,6 +485,7 @@ __global__ void ptc_sum_kernel(const double* partial, int n, double* out) {
 // c1 = 1 - beta1^t, c2 = 1 - beta2^t
 __global__ void ptc_adam_kernel(float* w, const double* g, float* m, float* v, int n, float lr, float b1,
                                 float b2, float eps, float c1, float c2) {
+  pdl_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float gr = 2.0f * (float)g[i];
@@ -491,9 +500,9 @@ __global__ void ptc_adam_kernel(float* w, const double* g, float* m, float* v, i
 template <int CIN, int COUT>
 void layer_r(int recon, const LayerArg& a, int npair, cudaStream_t st) {
   dim3 grid((2 * a.g.Vh + TPB - 1) / TPB, npair);
-  if (recon == 18) ptc_layer_kernel<CIN, COUT, 18><<<grid, TPB, 0, st>>>(a);
-  else if (recon == 12) ptc_layer_kernel<CIN, COUT, 12><<<grid, TPB, 0, st>>>(a);
-  else ptc_layer_kernel<CIN, COUT, 8><<<grid, TPB, 0, st>>>(a);
+  if (recon == 18) launch_pdl(ptc_layer_kernel<CIN, COUT, 18>, grid, TPB, 0, st, a);
+  else if (recon == 12) launch_pdl(ptc_layer_kernel<CIN, COUT, 12>, grid, TPB, 0, st, a);
+  else launch_pdl(ptc_layer_kernel<CIN, COUT, 8>, grid, TPB, 0, st, a);
 }
 template <int CIN>
 void layer_co(int cout, int recon, const LayerArg& a, int npair, cudaStream_t st) {
@@ -509,9 +518,9 @@ void launch_layer(int cin, int cout, int recon, const LayerArg& a, int npair, cu
 
 template <int CIN, int COUT>
 void wgrad_r(int recon, const GradArg& a, dim3 grid, cudaStream_t st) {
-  if (recon == 18) ptc_wgrad_kernel<CIN, COUT, 18><<<grid, WTPB, 0, st>>>(a);
-  else if (recon == 12) ptc_wgrad_kernel<CIN, COUT, 12><<<grid, WTPB, 0, st>>>(a);
-  else ptc_wgrad_kernel<CIN, COUT, 8><<<grid, WTPB, 0, st>>>(a);
+  if (recon == 18) launch_pdl(ptc_wgrad_kernel<CIN, COUT, 18>, grid, WTPB, 0, st, a);
+  else if (recon == 12) launch_pdl(ptc_wgrad_kernel<CIN, COUT, 12>, grid, WTPB, 0, st, a);
+  else launch_pdl(ptc_wgrad_kernel<CIN, COUT, 8>, grid, WTPB, 0, st, a);
 }
 template <int CIN>
 void wgrad_co(int cout, int recon, const GradArg& a, dim3 grid, cudaStream_t st) {
@@ -626,7 +635,7 @@ int wgrad(dirac_ptc* net, int l, char* const* x, char* const* gy, int npair, cud
   a.gauge = net->c->gauge[P32];
   a.g = geom(net);
   launch_wgrad(cin, cout, net->c->p.recon[P32], a, dim3(nblk, NPATH * na, npair), st);
-  ptc_wgrad_reduce<<<NPATH * cout * cin, dim3(32, RROWS), 0, st>>>(net->partial, nblk, npair, cout, cin,
+  launch_pdl(ptc_wgrad_reduce, NPATH * cout * cin, dim3(32, RROWS), 0, st, net->partial, nblk, npair, cout, cin,
                                                                  net->grad + 2 * net->woff[l - 1]);
   return DIRAC_OK;
 }
@@ -682,10 +691,10 @@ int forward_backward(dirac_ptc* n, const Work& W, const char* const* r, const ch
     gt.p[z * MAXC] = W.gra(L, z, 0);
   }
   double* part = n->dsc + DSC_PARTIAL;
-  ptc_norm_kernel<<<dim3(NORM_BLOCKS, B), GTPB, 0, st>>>(vt, n4, part);
-  ptc_inv_kernel<<<B, 32, 0, st>>>(part, NORM_BLOCKS, B, n->dsc);
-  ptc_loss_kernel<<<dim3(NORM_BLOCKS, B), GTPB, 0, st>>>(kt, vt, gt, n->dsc, n4, part);
-  ptc_sum_kernel<<<1, 32, 0, st>>>(part, NORM_BLOCKS * B, n->dsc + MAXB);
+  launch_pdl(ptc_norm_kernel, dim3(NORM_BLOCKS, B), GTPB, 0, st, vt, n4, part);
+  launch_pdl(ptc_inv_kernel, B, 32, 0, st, part, NORM_BLOCKS, B, n->dsc);
+  launch_pdl(ptc_loss_kernel, dim3(NORM_BLOCKS, B), GTPB, 0, st, kt, vt, gt, n->dsc, n4, part);
+  launch_pdl(ptc_sum_kernel, 1, 32, 0, st, part, NORM_BLOCKS * B, n->dsc + MAXB);
   if (!grads) return DIRAC_OK;
   for (int l = L; l >= 1; --l) {
     std::vector<char*> x(MAXB * MAXC), gy(MAXB * MAXC), gx(MAXB * MAXC);
@@ -701,7 +710,7 @@ int forward_backward(dirac_ptc* n, const Work& W, const char* const* r, const ch
     if (l > 1) {
       const int cin = n->ch[l - 1], cout = n->ch[l];
       const int nw = NPATH * cout * cin * 16;
-      ptc_adjoint_kernel<<<(nw + 127) / 128, 128, 0, st>>>(
+      launch_pdl(ptc_adjoint_kernel, (nw + 127) / 128, 128, 0, st, 
           reinterpret_cast<const float2*>(n->w) + n->woff[l - 1], reinterpret_cast<float2*>(n->wadj), cout, cin);
       run_layer(n, l, reinterpret_cast<const float2*>(n->wadj), cout, cin, gy.data(), gx.data(), B, st);
     }
@@ -967,7 +976,7 @@ extern "C" int dirac_ptc_train(dirac_ptc* n, const void* const* r, const void* c
     cudaMemcpyAsync(dloss + s, n->dsc + MAXB, sizeof(double), cudaMemcpyDeviceToDevice, st);
     n->t++;
     const double c1 = 1.0 - std::pow(P->beta1, (double)n->t), c2 = 1.0 - std::pow(P->beta2, (double)n->t);
-    ptc_adam_kernel<<<(nw2 + 255) / 256, 256, 0, st>>>(n->w, n->grad, n->am, n->av, nw2, (float)P->lr,
+    launch_pdl(ptc_adam_kernel, (nw2 + 255) / 256, 256, 0, st, n->w, n->grad, n->am, n->av, nw2, (float)P->lr,
                                                        (float)P->beta1, (float)P->beta2, (float)P->eps,
                                                        (float)c1, (float)c2);
   }

@@ -144,6 +144,7 @@ __device__ __forceinline__ void herm6_mac(const T* blk, const C<T> x[6], C<T> y[
 template <int PREC, int R>
 __global__ void __launch_bounds__(kMaxBlockSites, (SchwarzLayout<PREC, R>::kMinBlocks))
     schwarz_kernel(const SchwarzArg a) {
+  pdl_begin();
   using L = SchwarzLayout<PREC, R>;
   using T = typename L::T;
   using LIO = LinkIO<PREC, R>;
@@ -349,7 +350,7 @@ static int schwarz_launch(const SchwarzArg& a, int nblocks, int nbs, cudaStream_
       return DIRAC_ERR_CUDA;
     configured = true;
   }
-  kern<<<nblocks, threads, smem, st>>>(a);
+  launch_pdl(kern, nblocks, threads, smem, st, a);
   return cudaGetLastError() == cudaSuccess ? DIRAC_OK : DIRAC_ERR_CUDA;
 }
 

@@ -63,12 +63,14 @@ __device__ __forceinline__ void cdiv(double ar, double ai, double br, double bi,
 
 // --------------------------------------------------------------- scalar kernels
 __global__ void k_init(double* S) {
+  pdl_begin();
   for (int i = 0; i < S_END; ++i) S[i] = 0;
   S[S_ONE] = 1;
   S[S_RHOOLD] = 1; S[S_ALPHA] = 1; S[S_OMEGA] = 1;
 }
-__global__ void k_set(double* S, int slot, double v0, double v1) { S[slot] = v0; S[slot + 1] = v1; }
+__global__ void k_set(double* S, int slot, double v0, double v1) { pdl_begin(); S[slot] = v0; S[slot + 1] = v1; }
 __global__ void k_mirror(const double* S, int slot, double* mirror, int which, int it) {
+  pdl_begin();
   mirror[4 * which + 0] = S[slot];
   mirror[4 * which + 1] = S[S_FLAG];
   mirror[4 * which + 2] = it;
@@ -76,6 +78,7 @@ __global__ void k_mirror(const double* S, int slot, double* mirror, int which, i
 
 // BiCGstab: beta = (rho/rho_old)(alpha/omega); coefficient -beta*omega
 __global__ void k_bicg1(double* S) {
+  pdl_begin();
   double q1r, q1i, q2r, q2i;
   if (S[S_RHOOLD] == 0 && S[S_RHOOLD + 1] == 0) { flag(S, FLAG_BREAKDOWN); }
   if (S[S_OMEGA] == 0 && S[S_OMEGA + 1] == 0) { flag(S, FLAG_BREAKDOWN); }
@@ -92,6 +95,7 @@ __global__ void k_bicg1(double* S) {
 }
 // alpha = rho / (r0, v)
 __global__ void k_bicg2(double* S) {
+  pdl_begin();
   double sr = S[S_SIGMA], si = S[S_SIGMA + 1];
   if (bad(sr) || bad(si)) flag(S, FLAG_NONFINITE);
   else if (sr == 0 && si == 0) flag(S, FLAG_BREAKDOWN);
@@ -102,6 +106,7 @@ __global__ void k_bicg2(double* S) {
 }
 // omega = (t, s) / (t, t)
 __global__ void k_bicg3(double* S) {
+  pdl_begin();
   double tt = S[S_TS + 2];
   if (bad(tt) || bad(S[S_TS]) || bad(S[S_TS + 1])) flag(S, FLAG_NONFINITE);
   else if (tt == 0) flag(S, FLAG_BREAKDOWN);
@@ -112,6 +117,7 @@ __global__ void k_bicg3(double* S) {
 }
 // rho_old = rho; rho = (r0, r)
 __global__ void k_bicg4(double* S, double* mirror, int which, int it) {
+  pdl_begin();
   S[S_RHOOLD] = S[S_RHO]; S[S_RHOOLD + 1] = S[S_RHO + 1];
   S[S_RHO] = S[S_RN + 1]; S[S_RHO + 1] = S[S_RN + 2];
   if (bad(S[S_RN])) flag(S, FLAG_NONFINITE);
@@ -120,10 +126,11 @@ __global__ void k_bicg4(double* S, double* mirror, int which, int it) {
   mirror[4 * which + 2] = it;
 }
 // after a reliable update: rho = (r0, r) from a cdot into S_TMP
-__global__ void k_bicg_rho(double* S) { S[S_RHO] = S[S_TMP]; S[S_RHO + 1] = S[S_TMP + 1]; }
+__global__ void k_bicg_rho(double* S) { pdl_begin(); S[S_RHO] = S[S_TMP]; S[S_RHO + 1] = S[S_TMP + 1]; }
 
 // CG: alpha = rr / (p, Ap)
 __global__ void k_cg1(double* S) {
+  pdl_begin();
   double pap = S[S_PAP];
   if (bad(pap)) flag(S, FLAG_NONFINITE);
   else if (pap <= 0) flag(S, FLAG_BREAKDOWN);
@@ -133,6 +140,7 @@ __global__ void k_cg1(double* S) {
 }
 // beta = rr_new / rr
 __global__ void k_cg2(double* S, double* mirror, int which, int it) {
+  pdl_begin();
   double rn = S[S_RN];
   if (bad(rn)) flag(S, FLAG_NONFINITE);
   double b = (S[S_FLAG] == FLAG_OK && S[S_RR] > 0) ? rn / S[S_RR] : 0;
@@ -145,6 +153,7 @@ __global__ void k_cg2(double* S, double* mirror, int which, int it) {
 
 // GCR: gamma_k = ||z_k||, 1/gamma_k; move beta_{0,k} (a cdot result) into its slot
 __global__ void k_gcr_gamma(double* S, int k) {
+  pdl_begin();
   double zz = S[S_ZZ];
   if (bad(zz)) flag(S, FLAG_NONFINITE);
   else if (zz <= 0) flag(S, FLAG_BREAKDOWN);
@@ -159,6 +168,7 @@ __global__ void k_gcr_gamma(double* S, int k) {
 }
 // back-substitution of Algorithm 1: gamma_l chi_l + sum_{i>l} beta_{l,i} chi_i = alpha_l
 __global__ void k_gcr_backsub(double* S, int k) {
+  pdl_begin();
   for (int l = k - 1; l >= 0; --l) {
     double sr = S[S_GA + 4 * l], si = S[S_GA + 4 * l + 1];
     for (int i = l + 1; i < k; ++i) {
@@ -183,6 +193,7 @@ __global__ void k_gcr_backsub(double* S, int k) {
 // with zeta_{-1} = zeta_0 = 1, a_{-1} = 1, b_{-1} = 0.
 struct ShiftTable { double v[KSH]; };
 __global__ void k_ms_init(double* S, int n, ShiftTable sh) {
+  pdl_begin();
   for (int j = 0; j < KSH; ++j) {
     S[S_MSSH + j] = j < n ? sh.v[j] : 0;
     S[S_MSZ + j] = 1;
@@ -198,6 +209,7 @@ __global__ void k_ms_init(double* S, int n, ShiftTable sh) {
 }
 // base system: alpha = rr / (p, (A + sigma_0) p)
 __global__ void k_ms1(double* S) {
+  pdl_begin();
   double pap = S[S_PAP];
   if (bad(pap)) flag(S, FLAG_NONFINITE);
   else if (pap <= 0) flag(S, FLAG_BREAKDOWN);
@@ -207,6 +219,7 @@ __global__ void k_ms1(double* S) {
 }
 // every shift: zeta_{k+1}, a_j, b_j; retire systems that converged last time
 __global__ void k_ms2(double* S, int n, int j0, double tol2bb, double* mirror, int which, int it) {
+  pdl_begin();
   const double a = S[S_ALPHA], rr = S[S_RR], rn = S[S_RN];
   if (bad(rn)) flag(S, FLAG_NONFINITE);
   const double bk = (S[S_FLAG] == FLAG_OK && rr > 0) ? rn / rr : 0;
@@ -391,18 +404,18 @@ int solve_cg(Ctx& S, char* x, const char* b, const dirac_solver_params& P) {
   BT(blas_copy(B, S.f(rs, sp), S.f(r, P64), S.st));
   BT(blas_copy(B, S.f(p, sp), S.f(rs, sp), S.st));
   BT(blas_zero(B, S.f(xs, ap), S.st));
-  KC((k_init<<<1, 1, 0, S.st>>>(S.S)));
-  KC((k_set<<<1, 1, 0, S.st>>>(S.S, S_RR, rr, 0)));
+  KC((launch_pdl(k_init, 1, 1, 0, S.st, S.S)));
+  KC((launch_pdl(k_set, 1, 1, 0, S.st, S.S, S_RR, rr, 0)));
   double rmax = rr;
   int it = 0;
   bool converged = false;
   while (S.stats->iters < P.max_iter) {
     TRY(S.A(Ap, p, sp));
     BT(blas_cdot_norm(B, S.f(p, sp), S.f(Ap, sp), nullptr, S.st, S.slot(S_PAP)));
-    KC((k_cg1<<<1, 1, 0, S.st>>>(S.S)));
+    KC((launch_pdl(k_cg1, 1, 1, 0, S.st, S.S)));
     BT(blas_cg_update(B, cptr(S.slot(S_ALPHA)), S.f(p, sp), cptr(S.slot(S_NALPHA)), S.f(Ap, sp),
                       S.f(xs, ap), S.f(rs, sp), nullptr, S.st, S.slot(S_RN)));
-    KC((k_cg2<<<1, 1, 0, S.st>>>(S.S, S.mirror, it & 1, it)));
+    KC((launch_pdl(k_cg2, 1, 1, 0, S.st, S.S, S.mirror, it & 1, it)));
     BT(blas_axpby(B, cval(1), S.f(rs, sp), cptr(S.slot(S_BETA)), S.f(p, sp), S.st));
     TRY(S.mark(it));
     S.stats->iters++;
@@ -419,7 +432,7 @@ int solve_cg(Ctx& S, char* x, const char* b, const dirac_solver_params& P) {
         S.stats->reliable_updates++;
         if (rr < target) { converged = true; break; }
         BT(blas_copy(B, S.f(rs, sp), S.f(r, P64), S.st));
-        KC((k_set<<<1, 1, 0, S.st>>>(S.S, S_RR, rr, 0)));
+        KC((launch_pdl(k_set, 1, 1, 0, S.st, S.S, S_RR, rr, 0)));
         rmax = rr;
         it = -1;  // the mirror of the iteration before the update is stale
       }
@@ -508,7 +521,7 @@ int solve_bicgstab(Ctx& S, char* x, const char* b, const dirac_solver_params& P)
   BT(blas_zero(B, S.f(p, sp), S.st));
   BT(blas_zero(B, S.f(v, sp), S.st));
   BT(blas_zero(B, S.f(xs, ap), S.st));
-  KC((k_init<<<1, 1, 0, S.st>>>(S.S)));
+  KC((launch_pdl(k_init, 1, 1, 0, S.st, S.S)));
   BT(blas_cdot(B, S.f(r0, sp), S.f(rs, sp), nullptr, S.st, S.slot(S_RHO)));
   double rmax = rr;
   int it = 0;
@@ -516,22 +529,22 @@ int solve_bicgstab(Ctx& S, char* x, const char* b, const dirac_solver_params& P)
   // one iteration; its launches depend only on the mirror slot it & 1
   auto step = [&](int slot) -> int {
     Range range("BiCGstab iteration");
-    KC((k_bicg1<<<1, 1, 0, S.st>>>(S.S)));
+    KC((launch_pdl(k_bicg1, 1, 1, 0, S.st, S.S)));
     // p = r + beta (p - omega v)
     BT(blas_pupdate(B, S.f(rs, sp), cptr(S.slot(S_BETA)), cptr(S.slot(S_NBW)), S.f(v, sp), S.f(p, sp), S.st));
     TRY(S.A(v, p, sp));
     BT(blas_cdot(B, S.f(r0, sp), S.f(v, sp), nullptr, S.st, S.slot(S_SIGMA)));
-    KC((k_bicg2<<<1, 1, 0, S.st>>>(S.S)));
+    KC((launch_pdl(k_bicg2, 1, 1, 0, S.st, S.S)));
     // s = r - alpha v (in rs)
     BT(blas_caxpy_norm(B, cptr(S.slot(S_NALPHA)), S.f(v, sp), S.f(rs, sp), nullptr, S.st, S.slot(S_TMP)));
     TRY(S.A(t, rs, sp));
     BT(blas_cdot_norm(B, S.f(t, sp), S.f(rs, sp), nullptr, S.st, S.slot(S_TS)));
-    KC((k_bicg3<<<1, 1, 0, S.st>>>(S.S)));
+    KC((launch_pdl(k_bicg3, 1, 1, 0, S.st, S.S)));
     // xs += alpha p + omega s; r = s - omega t; ||r||^2, (r0, r)
     BT(blas_bicg_xr(B, cptr(S.slot(S_ALPHA)), S.f(p, sp), cptr(S.slot(S_OMEGA)), S.f(rs, sp),
                     cptr(S.slot(S_NOMEGA)), S.f(t, sp), S.f(xs, ap), S.f(r0, sp), nullptr, S.st,
                     S.slot(S_RN)));
-    KC((k_bicg4<<<1, 1, 0, S.st>>>(S.S, S.mirror, slot, slot)));
+    KC((launch_pdl(k_bicg4, 1, 1, 0, S.st, S.S, S.mirror, slot, slot)));
     return DIRAC_OK;
   };
   StepGraphs graphs(2, S.graphs);
@@ -552,7 +565,7 @@ int solve_bicgstab(Ctx& S, char* x, const char* b, const dirac_solver_params& P)
         if (rr < target) { converged = true; break; }
         BT(blas_copy(B, S.f(rs, sp), S.f(r, P64), S.st));
         BT(blas_cdot(B, S.f(r0, sp), S.f(rs, sp), nullptr, S.st, S.slot(S_TMP)));
-        KC((k_bicg_rho<<<1, 1, 0, S.st>>>(S.S)));
+        KC((launch_pdl(k_bicg_rho, 1, 1, 0, S.st, S.S)));
         rmax = rr;
         it = -1;
       }
@@ -647,7 +660,7 @@ int solve_gcr(Ctx& S, char* x, const char* b, const dirac_solver_params& P, int 
     kind = finite(red[1]) && red[1] < red[0] ? K_PTC : K_SCHWARZ;
   }
   S.stats->precond_kind = kind;
-  KC((k_init<<<1, 1, 0, S.st>>>(S.S)));
+  KC((launch_pdl(k_init, 1, 1, 0, S.st, S.S)));
   auto gb = [&](int i, int k) { return S.slot(S_GB + 4 * (i * KMAX + k) + 1); };
   // One GCR step at Krylov index k: p_k = K r_k, z_k = M p_k, orthogonalisation, the
   // residual update. Its launches depend only on k, so from the second restart cycle on
@@ -676,12 +689,12 @@ int solve_gcr(Ctx& S, char* x, const char* b, const dirac_solver_params& P, int 
       const double* blast = k == 1 ? S.slot(S_B0) : gb(k - 1, k);
       BT(blas_caxpy_norm(B, cptr(blast, -1), S.f(zv[k - 1], sp), S.f(zv[k], sp), nullptr, S.st, S.slot(S_ZZ)));
     }
-    KC((k_gcr_gamma<<<1, 1, 0, S.st>>>(S.S, k)));
+    KC((launch_pdl(k_gcr_gamma, 1, 1, 0, S.st, S.S, k)));
     // z_k /= gamma_k ; alpha_k = (z_k, r_k) ; r_{k+1} = r_k - alpha_k z_k
     BT(blas_scale_cdot(B, cptr(S.slot(S_INVG)), S.f(zv[k], sp), S.f(rh, sp), nullptr, S.st, S.slot(S_GA + 4 * k)));
     BT(blas_caxpy_norm(B, cptr(S.slot(S_GA + 4 * k), -1), S.f(zv[k], sp), S.f(rh, sp), nullptr, S.st,
                        S.slot(S_RH)));
-    KC((k_mirror<<<1, 1, 0, S.st>>>(S.S, S_RH, S.mirror, k & 1, k)));
+    KC((launch_pdl(k_mirror, 1, 1, 0, S.st, S.S, S_RH, S.mirror, k & 1, k)));
     return DIRAC_OK;
   };
   // Each preconditioner has its own captured steps. With K_SELECT (not forced) the choice
@@ -715,7 +728,7 @@ int solve_gcr(Ctx& S, char* x, const char* b, const dirac_solver_params& P, int 
       int fl;
       TRY(S.read(k - 1, &rp, &fl));
       if (fl != FLAG_OK) return flag_error(S, fl, "GCR");
-      KC((k_gcr_backsub<<<1, 1, 0, S.st>>>(S.S, k)));
+      KC((launch_pdl(k_gcr_backsub, 1, 1, 0, S.st, S.S, k)));
       std::vector<Cf> cf(k);
       std::vector<FieldRef> xs(k);
       for (int i = 0; i < k; ++i) {
@@ -786,8 +799,8 @@ int solve_ms_stage(Ctx& S, char* const* xout, const char* b, const double* shift
   }
   ShiftTable tab{};
   for (int j = 0; j < n; ++j) tab.v[j] = shifts[j];
-  KC((k_init<<<1, 1, 0, S.st>>>(S.S)));
-  KC((k_ms_init<<<1, 1, 0, S.st>>>(S.S, n, tab)));
+  KC((launch_pdl(k_init, 1, 1, 0, S.st, S.S)));
+  KC((launch_pdl(k_ms_init, 1, 1, 0, S.st, S.S, n, tab)));
   BT(blas_norm2(B, S.f(rs, sp), nullptr, S.st, S.slot(S_RR)));
   const double tol2bb = ms_tol * ms_tol * bb;
   S.shift = shifts[j0];
@@ -796,9 +809,9 @@ int solve_ms_stage(Ctx& S, char* const* xout, const char* b, const double* shift
     last = it;
     TRY(S.A(Ap, ps[j0].p, sp));
     BT(blas_cdot_norm(B, ps[j0], S.f(Ap, sp), nullptr, S.st, S.slot(S_PAP)));
-    KC((k_ms1<<<1, 1, 0, S.st>>>(S.S)));
+    KC((launch_pdl(k_ms1, 1, 1, 0, S.st, S.S)));
     BT(blas_caxpy_norm(B, cptr(S.slot(S_NALPHA)), S.f(Ap, sp), S.f(rs, sp), nullptr, S.st, S.slot(S_RN)));
-    KC((k_ms2<<<1, 1, 0, S.st>>>(S.S, n, j0, tol2bb, S.mirror, it & 1, it)));
+    KC((launch_pdl(k_ms2, 1, 1, 0, S.st, S.S, n, j0, tol2bb, S.mirror, it & 1, it)));
     BT(blas_multishift_update(B, n, xs.data(), ps.data(), S.f(rs, sp), S.slot(S_MSC), S.st));
     TRY(S.mark(it));
     S.stats->iters++;

@@ -185,6 +185,7 @@ __device__ __forceinline__ void stag_hop(const StagArg& a, const int x[4], int c
 // (2 to 3 of them in flight), which four lanes share.
 template <int PREC, int RL, int LANES>
 __global__ void __launch_bounds__(128) staggered_kernel(const StagArg a) {
+  pdl_begin();
   using T = typename Real<PREC>::T;
   const Geom& g = a.g;
   const int Vh = g.Vh;
@@ -271,9 +272,9 @@ template <int PREC, int LANES>
 static void launch_stag_lanes(int recon, const StagArg& a, cudaStream_t st) {
   const int per = 128 / LANES;
   dim3 block(128), grid((a.g.Vh + per - 1) / per);
-  if (recon == 18) staggered_kernel<PREC, 18, LANES><<<grid, block, 0, st>>>(a);
-  else if (recon == 12) staggered_kernel<PREC, 12, LANES><<<grid, block, 0, st>>>(a);
-  else staggered_kernel<PREC, 8, LANES><<<grid, block, 0, st>>>(a);
+  if (recon == 18) launch_pdl(staggered_kernel<PREC, 18, LANES>, grid, block, 0, st, a);
+  else if (recon == 12) launch_pdl(staggered_kernel<PREC, 12, LANES>, grid, block, 0, st, a);
+  else launch_pdl(staggered_kernel<PREC, 8, LANES>, grid, block, 0, st, a);
 }
 
 // Up to this many output sites four lanes share a site. Measured (two launches, us, one lane

@@ -579,6 +579,7 @@ __device__ __forceinline__ void wilson_site(const WilsonArg& a, int idx, size_t 
 template <int PREC, int R, bool FULLM>
 __global__ void __launch_bounds__(WilsonShape<PREC>::threads, WilsonShape<PREC>::minb)
     wilson_kernel(const WilsonArg a) {
+  pdl_begin();
   wilson_site<PREC, R, FULLM>(a, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
@@ -588,14 +589,14 @@ void launch_wilson_prec(int recon, bool fullm, const WilsonArg& a, cudaStream_t 
   constexpr int T = WilsonShape<PREC>::threads;
   dim3 block(T), grid((n + T - 1) / T);
   if (recon == 18) {
-    if (fullm) wilson_kernel<PREC, 18, true><<<grid, block, 0, st>>>(a);
-    else wilson_kernel<PREC, 18, false><<<grid, block, 0, st>>>(a);
+    if (fullm) launch_pdl(wilson_kernel<PREC, 18, true>, grid, block, 0, st, a);
+    else launch_pdl(wilson_kernel<PREC, 18, false>, grid, block, 0, st, a);
   } else if (recon == 12) {
-    if (fullm) wilson_kernel<PREC, 12, true><<<grid, block, 0, st>>>(a);
-    else wilson_kernel<PREC, 12, false><<<grid, block, 0, st>>>(a);
+    if (fullm) launch_pdl(wilson_kernel<PREC, 12, true>, grid, block, 0, st, a);
+    else launch_pdl(wilson_kernel<PREC, 12, false>, grid, block, 0, st, a);
   } else {
-    if (fullm) wilson_kernel<PREC, 8, true><<<grid, block, 0, st>>>(a);
-    else wilson_kernel<PREC, 8, false><<<grid, block, 0, st>>>(a);
+    if (fullm) launch_pdl(wilson_kernel<PREC, 8, true>, grid, block, 0, st, a);
+    else launch_pdl(wilson_kernel<PREC, 8, false>, grid, block, 0, st, a);
   }
 }
 

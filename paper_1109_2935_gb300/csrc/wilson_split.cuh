@@ -41,6 +41,7 @@ __device__ __forceinline__ C<double> row64(const char* m, int Vh, int cb, int bl
 
 template <int R, bool FULLM>
 __global__ void __launch_bounds__(32) wilson_split64_kernel(const WilsonArg a) {
+  pdl_begin();
   __shared__ double2 v[2][8][6];
   __shared__ double2 post[2][12];
   const Geom& g = a.g;
@@ -159,8 +160,8 @@ constexpr int kSplitSites = 8192;
 
 template <int R>
 static void launch_split64(bool fullm, const WilsonArg& a, int n, cudaStream_t st) {
-  if (fullm) wilson_split64_kernel<R, true><<<(n + 1) / 2, 32, 0, st>>>(a);
-  else wilson_split64_kernel<R, false><<<(n + 1) / 2, 32, 0, st>>>(a);
+  if (fullm) launch_pdl(wilson_split64_kernel<R, true>, (n + 1) / 2, 32, 0, st, a);
+  else launch_pdl(wilson_split64_kernel<R, false>, (n + 1) / 2, 32, 0, st, a);
 }
 
 // false: not launched (too many sites, or the hopping term is switched off)
