@@ -324,11 +324,11 @@ __device__ __forceinline__ void wilson_hop_h(C<float> acc[4][3], const float u[1
 
 // Launch shape per storage precision (threads per CTA, minimum resident CTAs per SM,
 // which caps registers). FP32/FP16 are memory-latency bound and want many warps in
-// flight; FP64 is FP64-ALU bound on this part.
-// Measured on GB300 at 24^3x128 (clover M, before the packed arithmetic): FP32 64x8 (128-register cap) 0.199 ms vs
-// 128x1 (up to 255 registers) 0.288 ms; FP16 ~0.178 ms for every shape tried.
-template <int PREC> struct WilsonShape { static constexpr int threads = 64, minb = 10; };
-template <> struct WilsonShape<P32> { static constexpr int threads = 64, minb = 8; };
+// flight, each with as many loads in flight as its registers hold; FP64 is FP64-ALU bound on
+// this part. Measured on GB300 at 24^3x128 (clover M): FP16 64 x 8 (128-register cap)
+// 135.2 us, 64 x 10 139.3, 64 x 12 138.6; FP32 64 x 8 190.6 us, before the packed arithmetic
+// 199 us against 288 us for 128 x 1 (up to 255 registers).
+template <int PREC> struct WilsonShape { static constexpr int threads = 64, minb = 8; };
 template <> struct WilsonShape<P64> { static constexpr int threads = 128, minb = 1; };
 template <> struct WilsonShape<P64DS> { static constexpr int threads = 128, minb = 2; };
 
