@@ -671,7 +671,7 @@ int solve_batched_impl(Run& R, const dirac_solver_params& P, dirac_solver_stats*
   launch_pdl(k_gather, (n + 63) / 64, 64, 0, R.st, R.scal, n, SC_BB, R.gathered());
   if (cudaStreamSynchronize(R.st) != cudaSuccess) return DIRAC_ERR_CUDA;
   std::vector<double> target(n), rmax(n), rr(n);
-  std::vector<int> active(n, 1), relup(n, 0), stale(n, 0);
+  std::vector<int> active(n, 1), relup(n, 0), stale(n, 0), settled(n, 0);
   for (int j = 0; j < n; ++j) R.upd_h()[j] = 1;  // the start covers every right-hand side
   for (int j = 0; j < n; ++j) {
     bb[j] = R.hgathered()[j];
@@ -783,7 +783,10 @@ int solve_batched_impl(Run& R, const dirac_solver_params& P, dirac_solver_stats*
             rr[j] = R.hgathered()[j];
             relup[j]++;
             stale[j] = 1;
-            if (rr[j] < target[j]) active[j] = 0;
+            if (rr[j] < target[j]) {
+              active[j] = 0;
+              settled[j] = 1;  // x and its FP64 residual are final
+            }
             rmax[j] = rr[j];
             R.active_h()[j] = active[j];
           }
@@ -798,16 +801,20 @@ int solve_batched_impl(Run& R, const dirac_solver_params& P, dirac_solver_stats*
     ++it;
   }
   if (rc == DIRAC_OK) {
-    // fold in what is left of the sloppy corrections and take the final FP64 residuals
-    // of every right-hand side
+    // fold in what is left of the sloppy corrections and take the final FP64 residuals of
+    // the right-hand sides that did not stop on theirs
+    bool left = false;
     if (cudaStreamSynchronize(R.st) != cudaSuccess) {
       rc = DIRAC_ERR_CUDA;
     } else {
-      for (int j = 0; j < n; ++j) R.upd_h()[j] = 1;
-      rc = reliable<SP, AP>(R, true);
+      for (int j = 0; j < n; ++j) {
+        R.upd_h()[j] = settled[j] ? 0 : 1;
+        left = left || !settled[j];
+      }
+      if (left) rc = reliable<SP, AP>(R, true);
     }
-    if (rc == DIRAC_OK)
-      for (int j = 0; j < n; ++j) rr[j] = R.hgathered()[j];
+    for (int j = 0; left && rc == DIRAC_OK && j < n; ++j)
+      if (!settled[j]) rr[j] = R.hgathered()[j];
   }
   for (int s = 0; s < 2; ++s) {
     if (graph[s]) cudaGraphExecDestroy(graph[s]);
