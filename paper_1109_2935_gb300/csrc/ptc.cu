@@ -557,6 +557,10 @@ struct dirac_ptc {
   float* partial = nullptr;
   size_t partial_bytes = 0;
   double* dsc = nullptr;   // [0, MAXB): inv; [MAXB]: loss; then norm / loss partials
+  char* tr = nullptr;      // training: sources r = M v made here (kept up to kKeepTrain bytes)
+  size_t tr_bytes = 0;
+  char* tl = nullptr;      // training: the loss of every step
+  size_t tl_bytes = 0;
   char* hid = nullptr;     // inference: two hidden-layer buffers of MAXC fields
   size_t fb = 0;           // bytes of one FP32 full field
   // tensor-core inference: BF16 weight images per layer, rebuilt after weight changes,
@@ -574,6 +578,7 @@ struct dirac_ptc {
 namespace dirac {
 namespace {
 
+constexpr size_t kKeepTrain = (size_t)256 << 20;
 constexpr int DSC_PARTIAL = MAXB + 8;
 constexpr int NORM_BLOCKS = 152;
 constexpr size_t DSC_DOUBLES = DSC_PARTIAL + (size_t)MAXB * NORM_BLOCKS;
@@ -794,6 +799,8 @@ void ptc_release(dirac_ptc* n) {
   cudaFree(n->act);
   cudaFree(n->partial);
   cudaFree(n->dsc);
+  cudaFree(n->tr);
+  cudaFree(n->tl);
   cudaFree(n->hid);
   cudaFree(n->tcimg);
   if (n->tc_err_h) cudaFreeHost(n->tc_err_h);
@@ -924,35 +931,21 @@ extern "C" int dirac_ptc_train(dirac_ptc* n, const void* const* r, const void* c
   cudaStream_t st = (cudaStream_t)stream;
   const int B = std::min(P->batch, npairs);
   // r_i = M v_i (FP32) when the caller gives only v
-  char* rbuf = nullptr;
+  // (a cudaMalloc and a cudaFree of both buffers per call cost a tenth of a short training)
   std::vector<const char*> rs(npairs);
   if (!r) {
-    if (cudaMalloc(&rbuf, (size_t)npairs * n->fb) != cudaSuccess) {
-      cudaGetLastError();
-      return net_err(n, DIRAC_ERR_OOM, "PTC training pairs");
-    }
+    if ((rc = grow(n, &n->tr, &n->tr_bytes, (size_t)npairs * n->fb))) return rc;
     for (int i = 0; i < npairs; ++i) {
-      if ((rc = apply_op(c, rbuf + (size_t)i * n->fb, (const char*)v[i], -1, P32, 0, st))) {
-        cudaFree(rbuf);
-        return rc;
-      }
-      rs[i] = rbuf + (size_t)i * n->fb;
+      if ((rc = apply_op(c, n->tr + (size_t)i * n->fb, (const char*)v[i], -1, P32, 0, st))) return rc;
+      rs[i] = n->tr + (size_t)i * n->fb;
     }
   } else {
     for (int i = 0; i < npairs; ++i) rs[i] = (const char*)r[i];
   }
-  double* dloss = nullptr;
-  if (P->steps > 0 && cudaMalloc(&dloss, P->steps * sizeof(double)) != cudaSuccess) {
-    cudaGetLastError();
-    cudaFree(rbuf);
-    return net_err(n, DIRAC_ERR_OOM, "PTC loss history");
-  }
+  if (P->steps > 0 && (rc = grow(n, &n->tl, &n->tl_bytes, P->steps * sizeof(double)))) return rc;
+  double* dloss = reinterpret_cast<double*>(n->tl);
   Work W;
-  if ((rc = make_work(n, B, &W))) {
-    cudaFree(rbuf);
-    cudaFree(dloss);
-    return rc;
-  }
+  if ((rc = make_work(n, B, &W))) return rc;
   // visiting order: Fisher-Yates shuffles of the pairs, one per epoch
   std::mt19937 gen(P->seed);
   std::vector<int> order(npairs);
@@ -985,8 +978,11 @@ extern "C" int dirac_ptc_train(dirac_ptc* n, const void* const* r, const void* c
       cudaMemcpy(loss, dloss, P->steps * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
     rc = cuda_check(c, "PTC train");
   cudaStreamSynchronize(st);
-  cudaFree(dloss);
-  cudaFree(rbuf);
+  if (n->tr_bytes > kKeepTrain) {
+    cudaFree(n->tr);
+    n->tr = nullptr;
+    n->tr_bytes = 0;
+  }
   if (rc == DIRAC_OK) rc = cuda_check(c, "PTC train");
   return rc;
 }
