@@ -13,6 +13,7 @@
 #include <type_traits>
 
 #include "internal.h"
+#include "solver_scalars.cuh"
 
 namespace dirac {
 
@@ -674,7 +675,7 @@ __device__ __forceinline__ void block_sum3(const double acc[3], RedShared& sh) {
 
 template <class Op>
 __global__ void __launch_bounds__(kThreads, MinBlocks<Op>::value) blas_reduce_kernel(Op op, int n, double* partials,
-                                                          unsigned* ticket, double* res) {
+                                                          unsigned* ticket, double* res, const Fin fin) {
   pdl_begin();
   __shared__ RedShared sh;
   double acc[3] = {0, 0, 0};
@@ -694,8 +695,13 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<Op>::value) blas_reduce_ke
 #pragma unroll
     for (int k = 0; k < 3; ++k) s[k] += __ldcg(partials + 3 * b + k);
   block_sum3(s, sh);
+  if (threadIdx.x >= 32) return;
   if (threadIdx.x < 3) res[threadIdx.x] = sh.sum[threadIdx.x];
-  if (threadIdx.x == 0) *ticket = 0;
+  __syncwarp();  // res is visible to thread 0
+  if (threadIdx.x == 0) {
+    *ticket = 0;
+    if (fin.op) run_fin(fin);
+  }
 }
 
 // ---------------------------------------------------------------- host dispatch
@@ -722,14 +728,14 @@ static int run_map(Blas* b, const Op& op, int n, cudaStream_t st) {
 
 template <class Op>
 static int run_reduce(Blas* b, const Op& op, int n, double* out, int nout, cudaStream_t st,
-                      double* dres) {
+                      double* dres, const Fin& fin = Fin{}) {
   // one wave of resident CTAs when the op asks for several per SM, else 4 per SM
   constexpr int kMaxGrid = MinBlocks<Op>::value > 1 ? 152 * MinBlocks<Op>::value : kRedBlocks;
   static_assert(kMaxGrid <= kRedBlocks, "partials buffer");
   int grid = (n + kThreads - 1) / kThreads;
   if (grid > kMaxGrid) grid = kMaxGrid;
   if (grid < 1) grid = 1;
-  launch_pdl(blas_reduce_kernel<Op>, grid, kThreads, 0, st, op, n, b->partials, b->ticket, dres ? dres : b->dev_res);
+  launch_pdl(blas_reduce_kernel<Op>, grid, kThreads, 0, st, op, n, b->partials, b->ticket, dres ? dres : b->dev_res, fin);
   int rc = check(b, "blas reduce kernel");
   if (rc || dres) return rc;  // device-resident result: no synchronisation
   cudaError_t e = cudaStreamSynchronize(st);
@@ -793,25 +799,25 @@ int blas_pupdate(Blas* b, const FieldRef& r, Cf beta, Cf c, const FieldRef& v, c
   if (all_h24({&r, &v, &p})) return run_map(b, (OpPUpdateH{r, v, p, beta, c}), nsites(p), st);
   DISPATCH(p, kind({&r, &v, &p}), return run_map(b, (OpPUpdate<NR, T>{r, v, p, beta, c}), NS, st));
 }
-int blas_norm2(Blas* b, const FieldRef& x, double* out, cudaStream_t st, double* dres) {
-  DISPATCH(x, kind({&x}), return run_reduce(b, (OpNorm2<NR, T>{x}), NS, out, 1, st, dres));
+int blas_norm2(Blas* b, const FieldRef& x, double* out, cudaStream_t st, double* dres, const Fin& fin) {
+  DISPATCH(x, kind({&x}), return run_reduce(b, (OpNorm2<NR, T>{x}), NS, out, 1, st, dres, fin));
 }
-int blas_cdot(Blas* b, const FieldRef& x, const FieldRef& y, double out[2], cudaStream_t st, double* dres) {
-  if (all_h24({&x, &y})) return run_reduce(b, (OpCdotNormH{x, y}), nsites(x), out, 2, st, dres);
+int blas_cdot(Blas* b, const FieldRef& x, const FieldRef& y, double out[2], cudaStream_t st, double* dres, const Fin& fin) {
+  if (all_h24({&x, &y})) return run_reduce(b, (OpCdotNormH{x, y}), nsites(x), out, 2, st, dres, fin);
   DISPATCH(x, kind({&x, &y}),
-           return run_reduce(b, (OpCdotNorm<NR, T>{x, y}), NS, out, 2, st, dres));
+           return run_reduce(b, (OpCdotNorm<NR, T>{x, y}), NS, out, 2, st, dres, fin));
 }
 int blas_cdot_norm(Blas* b, const FieldRef& x, const FieldRef& y, double out[3], cudaStream_t st,
-                   double* dres) {
-  if (all_h24({&x, &y})) return run_reduce(b, (OpCdotNormH{x, y}), nsites(x), out, 3, st, dres);
+                   double* dres, const Fin& fin) {
+  if (all_h24({&x, &y})) return run_reduce(b, (OpCdotNormH{x, y}), nsites(x), out, 3, st, dres, fin);
   DISPATCH(x, kind({&x, &y}),
-           return run_reduce(b, (OpCdotNorm<NR, T>{x, y}), NS, out, 3, st, dres));
+           return run_reduce(b, (OpCdotNorm<NR, T>{x, y}), NS, out, 3, st, dres, fin));
 }
 int blas_caxpy_norm(Blas* b, Cf a, const FieldRef& x, const FieldRef& y, double* out, cudaStream_t st,
-                    double* dres) {
-  if (all_h24({&x, &y})) return run_reduce(b, (OpCaxpyNormH<false>{x, y, y, a}), nsites(y), out, 1, st, dres);
+                    double* dres, const Fin& fin) {
+  if (all_h24({&x, &y})) return run_reduce(b, (OpCaxpyNormH<false>{x, y, y, a}), nsites(y), out, 1, st, dres, fin);
   DISPATCH(y, kind({&x, &y}),
-           return run_reduce(b, (OpCaxpyNorm<NR, T, false>{x, y, y, a}), NS, out, 1, st, dres));
+           return run_reduce(b, (OpCaxpyNorm<NR, T, false>{x, y, y, a}), NS, out, 1, st, dres, fin));
 }
 int blas_caxpy_norm_dot(Blas* b, Cf a, const FieldRef& x, const FieldRef& y, const FieldRef& w,
                         double out[3], cudaStream_t st, double* dres) {
@@ -820,16 +826,16 @@ int blas_caxpy_norm_dot(Blas* b, Cf a, const FieldRef& x, const FieldRef& y, con
            return run_reduce(b, (OpCaxpyNorm<NR, T, true>{x, y, w, a}), NS, out, 3, st, dres));
 }
 int blas_bicg_xr(Blas* b, Cf a, const FieldRef& p, Cf bb, const FieldRef& s, Cf c, const FieldRef& t,
-                 const FieldRef& xs, const FieldRef& w, double out[3], cudaStream_t st, double* dres) {
+                 const FieldRef& xs, const FieldRef& w, double out[3], cudaStream_t st, double* dres, const Fin& fin) {
   if (all_h24({&p, &s, &t, &w}) && xs.prec != P64 && xs.nr == 24)
-    return run_reduce(b, (OpBicgXRH{p, s, t, xs, w, a, bb, c}), nsites(s), out, 3, st, dres);
+    return run_reduce(b, (OpBicgXRH{p, s, t, xs, w, a, bb, c}), nsites(s), out, 3, st, dres, fin);
   DISPATCH(s, kind({&p, &s, &t, &xs, &w}),
-           return run_reduce(b, (OpBicgXR<NR, T>{p, s, t, xs, w, a, bb, c}), NS, out, 3, st, dres));
+           return run_reduce(b, (OpBicgXR<NR, T>{p, s, t, xs, w, a, bb, c}), NS, out, 3, st, dres, fin));
 }
 int blas_cg_update(Blas* b, Cf a, const FieldRef& p, Cf c, const FieldRef& Ap, const FieldRef& xs,
-                   const FieldRef& r, double* out, cudaStream_t st, double* dres) {
+                   const FieldRef& r, double* out, cudaStream_t st, double* dres, const Fin& fin) {
   DISPATCH(r, kind({&p, &Ap, &xs, &r}),
-           return run_reduce(b, (OpCgUpdate<NR, T>{p, Ap, xs, r, a, c}), NS, out, 1, st, dres));
+           return run_reduce(b, (OpCgUpdate<NR, T>{p, Ap, xs, r, a, c}), NS, out, 1, st, dres, fin));
 }
 int blas_scale_cdot(Blas* b, Cf s, const FieldRef& x, const FieldRef& y, double out[2], cudaStream_t st,
                     double* dres) {
@@ -1030,14 +1036,14 @@ extern "C" int dirac_cdot_noalloc(const void* x, const void* y, dirac_prec prec,
   const bool dbl = prec == DIRAC_PREC_F64;
   if (reals_per_site == 24) {
     if (dbl) blas_reduce_kernel<OpCdotNorm<24, double>><<<grid, kNoAllocThreads, 0, st>>>(
-        OpCdotNorm<24, double>{fx, fy}, (int)n, partials, ticket, result);
+        OpCdotNorm<24, double>{fx, fy}, (int)n, partials, ticket, result, Fin{});
     else blas_reduce_kernel<OpCdotNorm<24, float>><<<grid, kNoAllocThreads, 0, st>>>(
-        OpCdotNorm<24, float>{fx, fy}, (int)n, partials, ticket, result);
+        OpCdotNorm<24, float>{fx, fy}, (int)n, partials, ticket, result, Fin{});
   } else {
     if (dbl) blas_reduce_kernel<OpCdotNorm<6, double>><<<grid, kNoAllocThreads, 0, st>>>(
-        OpCdotNorm<6, double>{fx, fy}, (int)n, partials, ticket, result);
+        OpCdotNorm<6, double>{fx, fy}, (int)n, partials, ticket, result, Fin{});
     else blas_reduce_kernel<OpCdotNorm<6, float>><<<grid, kNoAllocThreads, 0, st>>>(
-        OpCdotNorm<6, float>{fx, fy}, (int)n, partials, ticket, result);
+        OpCdotNorm<6, float>{fx, fy}, (int)n, partials, ticket, result, Fin{});
   }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess)

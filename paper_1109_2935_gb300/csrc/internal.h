@@ -84,32 +84,39 @@ struct Blas;  // reduction scratch + pinned result slots
 Blas* blas_create();
 void blas_destroy(Blas*);
 // Reductions return their result on the host after a stream synchronisation, or, when
-// `dres` (3 doubles of device memory) is given, leave it there without synchronising.
+// `dres` (3 doubles of device memory) is given, leave it there without synchronising. Fin: a
+// solver's scalar step that the reduction runs once its result is in place
+// (solver_scalars.cuh).
+struct Fin {
+  int op = 0, a = 0, b = 0;
+  double* S = nullptr;
+  double* mirror = nullptr;
+};
 int blas_copy(Blas*, const FieldRef& dst, const FieldRef& src, cudaStream_t st);
 int blas_zero(Blas*, const FieldRef& x, cudaStream_t st);
 // y = a x + b y
 int blas_axpby(Blas*, Cf a, const FieldRef& x, Cf b, const FieldRef& y, cudaStream_t st);
 // p = r + b p + c v
 int blas_pupdate(Blas*, const FieldRef& r, Cf b, Cf c, const FieldRef& v, const FieldRef& p, cudaStream_t st);
-int blas_norm2(Blas*, const FieldRef& x, double* out, cudaStream_t st, double* dres = nullptr);
+int blas_norm2(Blas*, const FieldRef& x, double* out, cudaStream_t st, double* dres = nullptr, const Fin& fin = Fin{});
 int blas_cdot(Blas*, const FieldRef& x, const FieldRef& y, double out[2], cudaStream_t st,
-              double* dres = nullptr);
+              double* dres = nullptr, const Fin& fin = Fin{});
 // out = {Re (x,y), Im (x,y), ||x||^2}
 int blas_cdot_norm(Blas*, const FieldRef& x, const FieldRef& y, double out[3], cudaStream_t st,
-                   double* dres = nullptr);
+                   double* dres = nullptr, const Fin& fin = Fin{});
 // y += a x; out = ||y||^2
 int blas_caxpy_norm(Blas*, Cf a, const FieldRef& x, const FieldRef& y, double* out, cudaStream_t st,
-                    double* dres = nullptr);
+                    double* dres = nullptr, const Fin& fin = Fin{});
 // y += a x; out = {||y||^2, Re (w,y), Im (w,y)}
 int blas_caxpy_norm_dot(Blas*, Cf a, const FieldRef& x, const FieldRef& y, const FieldRef& w,
                         double out[3], cudaStream_t st, double* dres = nullptr);
 // xs += a p + b s; s += c t; out = {||s||^2, Re (w,s), Im (w,s)}
 int blas_bicg_xr(Blas*, Cf a, const FieldRef& p, Cf b, const FieldRef& s, Cf c, const FieldRef& t,
                  const FieldRef& xs, const FieldRef& w, double out[3], cudaStream_t st,
-                 double* dres = nullptr);
+                 double* dres = nullptr, const Fin& fin = Fin{});
 // xs += a p; r += c Ap; out = ||r||^2
 int blas_cg_update(Blas*, Cf a, const FieldRef& p, Cf c, const FieldRef& Ap, const FieldRef& xs,
-                   const FieldRef& r, double* out, cudaStream_t st, double* dres = nullptr);
+                   const FieldRef& r, double* out, cudaStream_t st, double* dres = nullptr, const Fin& fin = Fin{});
 // x *= Re s; out = (x, y) after scaling
 int blas_scale_cdot(Blas*, Cf s, const FieldRef& x, const FieldRef& y, double out[2], cudaStream_t st,
                     double* dres = nullptr);

@@ -19,6 +19,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "internal.h"
+#include "solver_scalars.cuh"
 
 namespace dirac {
 
@@ -32,36 +33,6 @@ struct Range {
 
 namespace {
 
-constexpr int KMAX = 20;
-// device scalar slots (doubles); every slot is 4 wide
-enum : int {
-  S_RHO = 0, S_RHOOLD = 4, S_ALPHA = 8, S_OMEGA = 12, S_SIGMA = 16, S_TS = 20, S_RN = 24,
-  S_BETA = 28, S_NBW = 32, S_NALPHA = 36, S_NOMEGA = 40, S_PAP = 44, S_RR = 48, S_ONE = 52,
-  S_FLAG = 56, S_TMP = 60, S_ZZ = 64, S_INVG = 68, S_B0 = 72, S_RH = 76,
-  S_GB = 128,                       // beta_{i,k}: slot (i * KMAX + k), value at +1, +2
-  S_GG = S_GB + 4 * KMAX * KMAX,    // gamma_k
-  S_GA = S_GG + 4 * KMAX,           // alpha_k (re, im)
-  S_GC = S_GA + 4 * KMAX,           // chi_k (re, im)
-  KSH = 16,                         // multi-shift: at most 16 shifts
-  S_MSC = S_GC + 4 * KMAX,          // per shift: a_j, zeta_{k+1,j}, b_j, active_j
-  S_MSZ = S_MSC + 4 * KSH,          // zeta_{k,j}
-  S_MSZP = S_MSZ + KSH,             // zeta_{k-1,j}
-  S_MSCV = S_MSZP + KSH,            // converged_j
-  S_MSSH = S_MSCV + KSH,            // sigma_j
-  S_MSAB = S_MSSH + KSH,            // a_{k-1}, b_{k-1} of the base system
-  S_END = S_MSAB + 4
-};
-enum : int { FLAG_OK = 0, FLAG_BREAKDOWN = 1, FLAG_NONFINITE = 2 };
-
-__device__ __forceinline__ bool bad(double v) { return !isfinite(v); }
-__device__ __forceinline__ void flag(double* S, int f) { if (S[S_FLAG] == FLAG_OK) S[S_FLAG] = f; }
-__device__ __forceinline__ void cdiv(double ar, double ai, double br, double bi, double& qr, double& qi) {
-  double d = br * br + bi * bi;
-  qr = (ar * br + ai * bi) / d;
-  qi = (ai * br - ar * bi) / d;
-}
-
-// --------------------------------------------------------------- scalar kernels
 __global__ void k_init(double* S) {
   pdl_begin();
   for (int i = 0; i < S_END; ++i) S[i] = 0;
@@ -69,12 +40,6 @@ __global__ void k_init(double* S) {
   S[S_RHOOLD] = 1; S[S_ALPHA] = 1; S[S_OMEGA] = 1;
 }
 __global__ void k_set(double* S, int slot, double v0, double v1) { pdl_begin(); S[slot] = v0; S[slot + 1] = v1; }
-__global__ void k_mirror(const double* S, int slot, double* mirror, int which, int it) {
-  pdl_begin();
-  mirror[4 * which + 0] = S[slot];
-  mirror[4 * which + 1] = S[S_FLAG];
-  mirror[4 * which + 2] = it;
-}
 
 // BiCGstab: beta = (rho/rho_old)(alpha/omega); coefficient -beta*omega
 __global__ void k_bicg1(double* S) {
@@ -93,79 +58,10 @@ __global__ void k_bicg1(double* S) {
   double wr = S[S_OMEGA], wi = S[S_OMEGA + 1];
   S[S_NBW] = -(br * wr - bi * wi); S[S_NBW + 1] = -(br * wi + bi * wr);
 }
-// alpha = rho / (r0, v)
-__global__ void k_bicg2(double* S) {
-  pdl_begin();
-  double sr = S[S_SIGMA], si = S[S_SIGMA + 1];
-  if (bad(sr) || bad(si)) flag(S, FLAG_NONFINITE);
-  else if (sr == 0 && si == 0) flag(S, FLAG_BREAKDOWN);
-  double ar = 0, ai = 0;
-  if (S[S_FLAG] == FLAG_OK) cdiv(S[S_RHO], S[S_RHO + 1], sr, si, ar, ai);
-  S[S_ALPHA] = ar; S[S_ALPHA + 1] = ai;
-  S[S_NALPHA] = -ar; S[S_NALPHA + 1] = -ai;
-}
-// omega = (t, s) / (t, t)
-__global__ void k_bicg3(double* S) {
-  pdl_begin();
-  double tt = S[S_TS + 2];
-  if (bad(tt) || bad(S[S_TS]) || bad(S[S_TS + 1])) flag(S, FLAG_NONFINITE);
-  else if (tt == 0) flag(S, FLAG_BREAKDOWN);
-  double wr = 0, wi = 0;
-  if (S[S_FLAG] == FLAG_OK) { wr = S[S_TS] / tt; wi = S[S_TS + 1] / tt; }
-  S[S_OMEGA] = S[S_FLAG] == FLAG_OK ? wr : 1; S[S_OMEGA + 1] = S[S_FLAG] == FLAG_OK ? wi : 0;
-  S[S_NOMEGA] = -wr; S[S_NOMEGA + 1] = -wi;
-}
-// rho_old = rho; rho = (r0, r)
-__global__ void k_bicg4(double* S, double* mirror, int which, int it) {
-  pdl_begin();
-  S[S_RHOOLD] = S[S_RHO]; S[S_RHOOLD + 1] = S[S_RHO + 1];
-  S[S_RHO] = S[S_RN + 1]; S[S_RHO + 1] = S[S_RN + 2];
-  if (bad(S[S_RN])) flag(S, FLAG_NONFINITE);
-  mirror[4 * which + 0] = S[S_RN];
-  mirror[4 * which + 1] = S[S_FLAG];
-  mirror[4 * which + 2] = it;
-}
 // after a reliable update: rho = (r0, r) from a cdot into S_TMP
 __global__ void k_bicg_rho(double* S) { pdl_begin(); S[S_RHO] = S[S_TMP]; S[S_RHO + 1] = S[S_TMP + 1]; }
 
-// CG: alpha = rr / (p, Ap)
-__global__ void k_cg1(double* S) {
-  pdl_begin();
-  double pap = S[S_PAP];
-  if (bad(pap)) flag(S, FLAG_NONFINITE);
-  else if (pap <= 0) flag(S, FLAG_BREAKDOWN);
-  double a = S[S_FLAG] == FLAG_OK ? S[S_RR] / pap : 0;
-  S[S_ALPHA] = a; S[S_ALPHA + 1] = 0;
-  S[S_NALPHA] = -a; S[S_NALPHA + 1] = 0;
-}
-// beta = rr_new / rr
-__global__ void k_cg2(double* S, double* mirror, int which, int it) {
-  pdl_begin();
-  double rn = S[S_RN];
-  if (bad(rn)) flag(S, FLAG_NONFINITE);
-  double b = (S[S_FLAG] == FLAG_OK && S[S_RR] > 0) ? rn / S[S_RR] : 0;
-  S[S_BETA] = b; S[S_BETA + 1] = 0;
-  if (S[S_FLAG] == FLAG_OK) S[S_RR] = rn;
-  mirror[4 * which + 0] = rn;
-  mirror[4 * which + 1] = S[S_FLAG];
-  mirror[4 * which + 2] = it;
-}
 
-// GCR: gamma_k = ||z_k||, 1/gamma_k; move beta_{0,k} (a cdot result) into its slot
-__global__ void k_gcr_gamma(double* S, int k) {
-  pdl_begin();
-  double zz = S[S_ZZ];
-  if (bad(zz)) flag(S, FLAG_NONFINITE);
-  else if (zz <= 0) flag(S, FLAG_BREAKDOWN);
-  double g = S[S_FLAG] == FLAG_OK ? sqrt(zz) : 1;
-  S[S_GG + 4 * k] = g;
-  S[S_INVG] = S[S_FLAG] == FLAG_OK ? 1.0 / g : 0;
-  S[S_INVG + 1] = 0;
-  if (k > 0) {
-    S[S_GB + 4 * (0 * KMAX + k) + 1] = S[S_B0];
-    S[S_GB + 4 * (0 * KMAX + k) + 2] = S[S_B0 + 1];
-  }
-}
 // back-substitution of Algorithm 1: gamma_l chi_l + sum_{i>l} beta_{l,i} chi_i = alpha_l
 __global__ void k_gcr_backsub(double* S, int k) {
   pdl_begin();
@@ -306,6 +202,7 @@ struct Ctx {
     return apply_op(c, out, in, parity, prec, which, st, which == 2 ? shift : 0.0);
   }
   double* slot(int s) const { return S + s; }
+  Fin fin(int op, int a = 0, int b = 0) const { return Fin{op, a, b, S, mirror}; }
   // record the end of iteration `it`; its mirror entry is it % 2
   int mark(int it) { return cudaEventRecord(ev[it & 1], st) == cudaSuccess ? DIRAC_OK : DIRAC_ERR_CUDA; }
   // wait for iteration `it` and return its mirrored {value, flag}
@@ -416,11 +313,9 @@ int solve_cg(Ctx& S, char* x, const char* b, const dirac_solver_params& P) {
   bool converged = false;
   while (S.stats->iters < P.max_iter) {
     TRY(S.A(Ap, p, sp));
-    BT(blas_cdot_norm(B, S.f(p, sp), S.f(Ap, sp), nullptr, S.st, S.slot(S_PAP)));
-    KC((launch_pdl(k_cg1, 1, 1, 0, S.st, S.S)));
+    BT(blas_cdot_norm(B, S.f(p, sp), S.f(Ap, sp), nullptr, S.st, S.slot(S_PAP), S.fin(FIN_CG1)));
     BT(blas_cg_update(B, cptr(S.slot(S_ALPHA)), S.f(p, sp), cptr(S.slot(S_NALPHA)), S.f(Ap, sp),
-                      S.f(xs, ap), S.f(rs, sp), nullptr, S.st, S.slot(S_RN)));
-    KC((launch_pdl(k_cg2, 1, 1, 0, S.st, S.S, S.mirror, it & 1, it)));
+                      S.f(xs, ap), S.f(rs, sp), nullptr, S.st, S.slot(S_RN), S.fin(FIN_CG2, 0, it)));
     BT(blas_axpby(B, cval(1), S.f(rs, sp), cptr(S.slot(S_BETA)), S.f(p, sp), S.st));
     TRY(S.mark(it));
     S.stats->iters++;
@@ -544,18 +439,15 @@ int solve_bicgstab(Ctx& S, char* x, const char* b, const dirac_solver_params& P)
     // p = r + beta (p - omega v)
     BT(blas_pupdate(B, S.f(rs, sp), cptr(S.slot(S_BETA)), cptr(S.slot(S_NBW)), S.f(v, sp), S.f(p, sp), S.st));
     TRY(S.A(v, p, sp));
-    BT(blas_cdot(B, S.f(r0, sp), S.f(v, sp), nullptr, S.st, S.slot(S_SIGMA)));
-    KC((launch_pdl(k_bicg2, 1, 1, 0, S.st, S.S)));
+    BT(blas_cdot(B, S.f(r0, sp), S.f(v, sp), nullptr, S.st, S.slot(S_SIGMA), S.fin(FIN_BICG2)));
     // s = r - alpha v (in rs)
     BT(blas_caxpy_norm(B, cptr(S.slot(S_NALPHA)), S.f(v, sp), S.f(rs, sp), nullptr, S.st, S.slot(S_TMP)));
     TRY(S.A(t, rs, sp));
-    BT(blas_cdot_norm(B, S.f(t, sp), S.f(rs, sp), nullptr, S.st, S.slot(S_TS)));
-    KC((launch_pdl(k_bicg3, 1, 1, 0, S.st, S.S)));
+    BT(blas_cdot_norm(B, S.f(t, sp), S.f(rs, sp), nullptr, S.st, S.slot(S_TS), S.fin(FIN_BICG3)));
     // xs += alpha p + omega s; r = s - omega t; ||r||^2, (r0, r)
     BT(blas_bicg_xr(B, cptr(S.slot(S_ALPHA)), S.f(p, sp), cptr(S.slot(S_OMEGA)), S.f(rs, sp),
                     cptr(S.slot(S_NOMEGA)), S.f(t, sp), S.f(xs, ap), S.f(r0, sp), nullptr, S.st,
-                    S.slot(S_RN)));
-    KC((launch_pdl(k_bicg4, 1, 1, 0, S.st, S.S, S.mirror, slot, slot)));
+                    S.slot(S_RN), S.fin(FIN_BICG4, 0, slot)));
     return DIRAC_OK;
   };
   StepGraphs graphs(2, S.graphs);
@@ -695,7 +587,7 @@ int solve_gcr(Ctx& S, char* x, const char* b, const dirac_solver_params& P, int 
     // modified Gram-Schmidt: beta_ik = (z_i, z_k); z_k -= beta_ik z_i. Each pass
     // subtracts the previous projection and forms the next inner product.
     if (k == 0) {
-      BT(blas_norm2(B, S.f(zv[0], sp), nullptr, S.st, S.slot(S_ZZ)));
+      BT(blas_norm2(B, S.f(zv[0], sp), nullptr, S.st, S.slot(S_ZZ), S.fin(FIN_GCR_GAMMA, k)));
     } else {
       BT(blas_cdot(B, S.f(zv[0], sp), S.f(zv[k], sp), nullptr, S.st, S.slot(S_B0)));
       for (int i = 1; i < k; ++i) {
@@ -704,14 +596,13 @@ int solve_gcr(Ctx& S, char* x, const char* b, const dirac_solver_params& P, int 
                                nullptr, S.st, gb(i, k) - 1));
       }
       const double* blast = k == 1 ? S.slot(S_B0) : gb(k - 1, k);
-      BT(blas_caxpy_norm(B, cptr(blast, -1), S.f(zv[k - 1], sp), S.f(zv[k], sp), nullptr, S.st, S.slot(S_ZZ)));
+      BT(blas_caxpy_norm(B, cptr(blast, -1), S.f(zv[k - 1], sp), S.f(zv[k], sp), nullptr, S.st, S.slot(S_ZZ),
+                         S.fin(FIN_GCR_GAMMA, k)));
     }
-    KC((launch_pdl(k_gcr_gamma, 1, 1, 0, S.st, S.S, k)));
     // z_k /= gamma_k ; alpha_k = (z_k, r_k) ; r_{k+1} = r_k - alpha_k z_k
     BT(blas_scale_cdot(B, cptr(S.slot(S_INVG)), S.f(zv[k], sp), S.f(rh, sp), nullptr, S.st, S.slot(S_GA + 4 * k)));
     BT(blas_caxpy_norm(B, cptr(S.slot(S_GA + 4 * k), -1), S.f(zv[k], sp), S.f(rh, sp), nullptr, S.st,
-                       S.slot(S_RH)));
-    KC((launch_pdl(k_mirror, 1, 1, 0, S.st, S.S, S_RH, S.mirror, k & 1, k)));
+                       S.slot(S_RH), S.fin(FIN_MIRROR, S_RH, k)));
     return DIRAC_OK;
   };
   // Each preconditioner has its own captured steps. With K_SELECT (not forced) the choice
