@@ -45,7 +45,7 @@ struct BatchLat {
 
 // output site idx of right-hand sides rhs .. rhs + N - 1
 template <int PREC, int R, int N = 1>
-__device__ __forceinline__ void batch_site(const BatchLat& L, int rhs, int idx) {
+__device__ __forceinline__ void batch_site(const BatchLat& L, int rhs, int idx, char* ring = nullptr) {
   WilsonArg a;
   a.g = L.g;
   a.gauge = L.gauge;
@@ -60,7 +60,7 @@ __device__ __forceinline__ void batch_site(const BatchLat& L, int rhs, int idx) 
   a.in[1] = in + hb;
   a.out[0] = out;
   a.out[1] = out + hb;
-  wilson_site<PREC, R, true, N>(a, idx, L.field_bytes);
+  wilson_site<PREC, R, true, N>(a, idx, L.field_bytes, ring);
 }
 
 // Tile t of lattice L: warp y of the CTA has right-hand sides y NR .. y NR + NR - 1 of the
@@ -77,7 +77,7 @@ __device__ __forceinline__ void batch_tile(const BatchLat& L, int t, int RG) {
   if constexpr (NR == 2) {
     const bool second = on(rhs + 1);
     if (first && second) {
-      batch_site<PREC, R, 2>(L, rhs, idx);
+      batch_site<PREC, R, 2>(L, rhs, idx, ring_of_warp<PREC, R, 2>(y));
       return;
     }
     if (!first && !second) return;
@@ -189,9 +189,9 @@ __global__ void __launch_bounds__(kTileSites * 4, 1)
 template <int PREC, int NR>
 static void launch_mrhs_prec(int recon, const BatchLat& L, int RG, int grid, cudaStream_t st) {
   dim3 block(kTileSites, RG / NR);
-  if (recon == 18) launch_pdl(mrhs_kernel<PREC, 18, NR>, grid, block, 0, st, L, RG);
-  else if (recon == 12) launch_pdl(mrhs_kernel<PREC, 12, NR>, grid, block, 0, st, L, RG);
-  else launch_pdl(mrhs_kernel<PREC, 8, NR>, grid, block, 0, st, L, RG);
+  if (recon == 18) launch_pdl(mrhs_kernel<PREC, 18, NR>, grid, block, RG / NR * kRingWarp<PREC, 18, NR>, st, L, RG);
+  else if (recon == 12) launch_pdl(mrhs_kernel<PREC, 12, NR>, grid, block, RG / NR * kRingWarp<PREC, 12, NR>, st, L, RG);
+  else launch_pdl(mrhs_kernel<PREC, 8, NR>, grid, block, RG / NR * kRingWarp<PREC, 8, NR>, st, L, RG);
 }
 template <int PREC, int NR>
 static void launch_batch_prec(int recon, const std::vector<BatchLat>& l, int ntiles, int RG, int grid, cudaStream_t st) {
@@ -199,9 +199,9 @@ static void launch_batch_prec(int recon, const std::vector<BatchLat>& l, int nti
   for (size_t k = 0; k < l.size(); ++k) t.v[k] = l[k];
   const int nlat = (int)l.size();
   dim3 block(kTileSites, RG / NR);
-  if (recon == 18) batch_kernel<PREC, 18, NR><<<grid, block, 0, st>>>(t, nlat, ntiles, RG);
-  else if (recon == 12) batch_kernel<PREC, 12, NR><<<grid, block, 0, st>>>(t, nlat, ntiles, RG);
-  else batch_kernel<PREC, 8, NR><<<grid, block, 0, st>>>(t, nlat, ntiles, RG);
+  if (recon == 18) batch_kernel<PREC, 18, NR><<<grid, block, (RG / NR * kRingWarp<PREC, 18, NR>), st>>>(t, nlat, ntiles, RG);
+  else if (recon == 12) batch_kernel<PREC, 12, NR><<<grid, block, (RG / NR * kRingWarp<PREC, 12, NR>), st>>>(t, nlat, ntiles, RG);
+  else batch_kernel<PREC, 8, NR><<<grid, block, (RG / NR * kRingWarp<PREC, 8, NR>), st>>>(t, nlat, ntiles, RG);
 }
 
 static void launch_batch64(int recon, const BatchLat* d, int nlat, int nrhs, int grid, cudaStream_t st) {
