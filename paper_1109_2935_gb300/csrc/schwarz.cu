@@ -12,9 +12,9 @@
 // FP32/FP16 storage: the block's forward links and clover are copied into shared
 // memory in their storage format (raw chunks: binary16 stays binary16, so an FP16
 // block needs 87 KB and two CTAs fit on an SM) and decoded on use; the clover's FP16
-// per-site norm scales the 6-component input instead of the 36 entries. The hopping
-// sum is accumulated unscaled and multiplied by -kappa once, only a wrapping t hop
-// with antiperiodic time taking its sign. The residual r lives in shared memory in
+// per-site norm scales the 6-component input instead of the 36 entries. -kappa (and the
+// sign of a wrapping t hop with antiperiodic time) is the factor of each hop's fused
+// accumulation, so it costs no instruction. The residual r lives in shared memory in
 // FP32, x in registers; reductions are warp shuffles plus one shared-memory stage.
 // FP64 storage: r in shared memory, links and clover read through the read-only cache.
 #include "internal.h"
@@ -181,10 +181,11 @@ __global__ void __launch_bounds__(kMaxBlockSites, (SchwarzLayout<PREC, R>::kMinB
   const size_t hb = SpinorIO<PREC, 24>::half_bytes(Vh);
   const char* clov_g = a.clover + par * CloverIO<PREC>::parity_bytes(Vh);
 
-  // neighbour local indices, -1 where the hop leaves the block, and the sign of the
-  // two t hops (-1 for a wrapping hop with antiperiodic time)
+  // neighbour local indices, -1 where the hop leaves the block, and the factor of the
+  // two t hops (sign flipped for a wrapping hop with antiperiodic time)
   int nbr[8];
-  T tsign[2] = {(T)1, (T)1};
+  const T mk = (T)(-a.kappa);  // multiplies every hop's accumulation
+  T tsign[2] = {mk, mk};
   {
     int stride = 1;
 #pragma unroll
@@ -196,7 +197,7 @@ __global__ void __launch_bounds__(kMaxBlockSites, (SchwarzLayout<PREC, R>::kMinB
         if (ln == a.b[mu] || ln < 0) {
           if (a.b[mu] != g.L[mu]) ok = false;
           ln = dir == 0 ? 0 : a.b[mu] - 1;
-          if (mu == 3 && g.apbc) tsign[dir] = (T)-1;
+          if (mu == 3 && g.apbc) tsign[dir] = -mk;
         }
         nbr[2 * mu + dir] = ok ? t + (ln - l[mu]) * stride : -1;
       }
@@ -233,12 +234,11 @@ __global__ void __launch_bounds__(kMaxBlockSites, (SchwarzLayout<PREC, R>::kMinB
   }
   __syncthreads();
 
-  const T mk = (T)(-a.kappa);
   for (int step = 0; step < a.steps; ++step) {
     T p[24];
     T red3[3] = {0, 0, 0};
     if (active) {
-      // p = Ahat r - kappa D_B r on this site: the hopping sum first, unscaled
+      // p = Ahat r - kappa D_B r on this site: the hopping sum first
       C<T> acc[4][3];
 #pragma unroll
       for (int s = 0; s < 4; ++s)
@@ -267,16 +267,12 @@ __global__ void __launch_bounds__(kMaxBlockSites, (SchwarzLayout<PREC, R>::kMinB
             }
           }
           const T s = dir == 0 ? (T)-1 : (T)1;
-          if (mu == 0) wilson_hop<0>(acc, psi, U, dir == 1, s, (T)1);
-          if (mu == 1) wilson_hop<1>(acc, psi, U, dir == 1, s, (T)1);
-          if (mu == 2) wilson_hop<2>(acc, psi, U, dir == 1, s, (T)1);
+          if (mu == 0) wilson_hop<0>(acc, psi, U, dir == 1, s, mk);
+          if (mu == 1) wilson_hop<1>(acc, psi, U, dir == 1, s, mk);
+          if (mu == 2) wilson_hop<2>(acc, psi, U, dir == 1, s, mk);
           if (mu == 3) wilson_hop<3>(acc, psi, U, dir == 1, s, tsign[dir]);
         }
       }
-#pragma unroll
-      for (int s = 0; s < 4; ++s)
-#pragma unroll
-        for (int c = 0; c < 3; ++c) acc[s][c] = C<T>{mk * acc[s][c].r, mk * acc[s][c].i};
       // + Ahat r, chirality block by block; the FP16 norm scales the 6-component input
 #pragma unroll
       for (int blk = 0; blk < 2; ++blk) {
