@@ -338,15 +338,26 @@ template <int SP> struct OpShadow {  // r0 = rs
     store_v<SP>(g, VR0, r, s, u);
   }
 };
-template <int SP, int AP> struct OpRestart {  // rs = r (sloppy); xs = 0
-  static constexpr int NRED = 0, OUT = 0;
-  __device__ void operator()(const Seg& g, int r, int s, const double*, double*) const {
-    double y[24], z[24];
+// rs = r (sloppy), then (r0, rs) of the values as stored; xs is already 0 (OpInit, OpXUpd)
+template <int SP> struct OpRestart {
+  static constexpr int NRED = 2, OUT = SC_TMP;
+  using T = typename Real<SP>::T;
+  __device__ void operator()(const Seg& g, int r, int s, const double*, double* acc) const {
+    double y[24];
+    T u[24], z[24];
     load_v<P64>(g, VR, r, s, y);
-    store_v<SP>(g, VRS, r, s, y);
+    load_v<SP>(g, VR0, r, s, z);
 #pragma unroll
-    for (int k = 0; k < 24; ++k) z[k] = 0;
-    store_v<AP>(g, VXS, r, s, z);
+    for (int k = 0; k < 24; ++k) u[k] = (T)y[k];
+    store_q<SP>(g, VRS, r, s, u);
+    T re = 0, im = 0;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      re += z[2 * k] * u[2 * k] + z[2 * k + 1] * u[2 * k + 1];
+      im += z[2 * k] * u[2 * k + 1] - z[2 * k + 1] * u[2 * k];
+    }
+    acc[0] += re;
+    acc[1] += im;
   }
 };
 
@@ -654,8 +665,7 @@ int reliable(Run& R, bool exact) {
 }
 template <int SP, int AP>
 int restart(Run& R, int first) {
-  RT(launch(R, OpRestart<SP, AP>{}, UPDATING));
-  RT(launch(R, OpCdot<SP, VR0, VRS, SC_TMP>{}, UPDATING));
+  RT(launch(R, OpRestart<SP>{}, UPDATING));
   // the host's active flags (pinned, mapped) for the scalar state
   launch_pdl(k_restart, (R.nrhs + 63) / 64, 64, 0, R.st, R.scal, R.nrhs, R.active_d(), R.upd_d(), first);
   return cudaGetLastError() == cudaSuccess ? DIRAC_OK : DIRAC_ERR_CUDA;
@@ -686,7 +696,7 @@ int solve_batched_impl(Run& R, const dirac_solver_params& P, dirac_solver_stats*
     RT(launch(R, OpInit<SP, AP, true>{}));
     RT(dirac_batch_apply(R.plan_x, R.st));
     RT(launch(R, OpXmy{}));
-    RT(launch(R, OpRestart<SP, AP>{}));
+    RT(launch(R, OpRestart<SP>{}));
     RT(launch(R, OpShadow<SP>{}));
     launch_pdl(k_gather, (n + 63) / 64, 64, 0, R.st, R.scal, n, SC_RR, R.gathered());
     if (cudaStreamSynchronize(R.st) != cudaSuccess) return DIRAC_ERR_CUDA;
