@@ -236,8 +236,7 @@ __global__ void __launch_bounds__(TPB, CIN * COUT <= 4 ? 4 : 1) ptc_layer_kernel
 // path is made once per site and block and shared by the N = max(c_in, c_out) contractions:
 // with c_in <= c_out, a block has one input channel a, transports it (t) and contracts it
 // with every g_c; otherwise it has one output channel a and moves the link to the other
-// factor, sum_colour g (U f)^dagger = (U^dagger g) f^dagger. FP32-bound like the layer; one
-// wave of blocks, so that the block sums at the end stay a few percent. Measured on the
+// factor, sum_colour g (U f)^dagger = (U^dagger g) f^dagger. FP32-bound like the layer. Measured on the
 // (2, 2) layer, 16^4 x 4 pairs: 270 us with a transport per (c_in, c_out).
 constexpr int WTPB = 128;  // threads per block
 constexpr int wgrad_ctas(int n) { return n == 1 ? 4 : n == 2 ? 3 : 2; }  // blocks per SM (registers)
@@ -627,7 +626,9 @@ int wgrad(dirac_ptc* net, int l, char* const* x, char* const* gy, int npair, cud
   const int Vh = net->c->g.Vh;
   const int na = std::min(cin, cout), n = std::max(cin, cout);
   const int maxblk = (2 * Vh + WTPB - 1) / WTPB;
-  const int nblk = std::max(1, std::min(152 * wgrad_ctas(n) / (NPATH * na * npair), maxblk));
+  // 16 sites or so per thread at 16^4 x 4 pairs: a thread's FP32 chain is what limits the
+  // gradient's accuracy (85 sites, one wave of blocks, lost a factor of 2.5)
+  const int nblk = std::max(1, std::min(2 * ((152 * 8 + NPATH * cout * npair - 1) / (NPATH * cout * npair)), maxblk));
   size_t need = (size_t)npair * NPATH * na * nblk * n * 32 * sizeof(float);
   int rc = grow(net, reinterpret_cast<char**>(&net->partial), &net->partial_bytes, need);
   if (rc) return rc;
