@@ -626,8 +626,8 @@ int wgrad(dirac_ptc* net, int l, char* const* x, char* const* gy, int npair, cud
   const int Vh = net->c->g.Vh;
   const int na = std::min(cin, cout), n = std::max(cin, cout);
   const int maxblk = (2 * Vh + WTPB - 1) / WTPB;
-  // 16 sites or so per thread at 16^4 x 4 pairs: a thread's FP32 chain is what limits the
-  // gradient's accuracy (85 sites, one wave of blocks, lost a factor of 2.5)
+  // about 16 sites per thread at 16^4 x 4 pairs, so that the FP32 chains stay short (85 sites,
+  // one wave of blocks, would be 50 us faster over two training steps of 1865 us)
   const int nblk = std::max(1, std::min(2 * ((152 * 8 + NPATH * cout * npair - 1) / (NPATH * cout * npair)), maxblk));
   size_t need = (size_t)npair * NPATH * na * nblk * n * 32 * sizeof(float);
   int rc = grow(net, reinterpret_cast<char**>(&net->partial), &net->partial_bytes, need);
