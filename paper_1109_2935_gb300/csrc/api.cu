@@ -340,6 +340,7 @@ int dirac_load_gauge(dirac_ctx* c, const double* links, int which, int on_device
       rc = cuda_check(c, "build clover");
     }
   }
+  launch_settle(st);
   if (staging) {
     cudaStreamSynchronize(st);
     cudaFree(staging);

@@ -60,17 +60,17 @@ __device__ __forceinline__ void any_load(const FieldRef& f, int s, T v[NR]) {
   const char* b = f.p + q * f.hb;
   if (f.prec == P64) {
     double t[NR];
-    SpinorIO<P64, NR>::template load<false>(b, f.Vh, cb, t);
+    SpinorIO<P64, NR>::load(b, f.Vh, cb, t);
 #pragma unroll
     for (int k = 0; k < NR; ++k) v[k] = (T)t[k];
   } else if (f.prec == P32) {
     float t[NR];
-    SpinorIO<P32, NR>::template load<false>(b, f.Vh, cb, t);
+    SpinorIO<P32, NR>::load(b, f.Vh, cb, t);
 #pragma unroll
     for (int k = 0; k < NR; ++k) v[k] = (T)t[k];
   } else {
     float t[NR];
-    SpinorIO<P16, NR>::template load<false>(b, f.Vh, cb, t);
+    SpinorIO<P16, NR>::load(b, f.Vh, cb, t);
 #pragma unroll
     for (int k = 0; k < NR; ++k) v[k] = (T)t[k];
   }

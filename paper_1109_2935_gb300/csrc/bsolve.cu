@@ -61,7 +61,7 @@ __device__ __forceinline__ void load_v(const Seg& g, int v, int r, int s, T out[
   int cb;
   const char* b = site_base(g, v, r, s, cb);
   typename Real<PREC>::T t[24];
-  SpinorIO<PREC, 24>::template load<false>(b, g.Vh, cb, t);
+  SpinorIO<PREC, 24>::load(b, g.Vh, cb, t);
 #pragma unroll
   for (int k = 0; k < 24; ++k) out[k] = (T)t[k];
 }

@@ -208,14 +208,21 @@ __device__ __forceinline__ float fma_hh(uint32_t a, uint32_t b, float c) {
 template <int BYTES> __device__ __forceinline__ const char* chunk_at(const char* b, int k, int Vh, int cb) {
   return b + (size_t)k * Vh * BYTES + (size_t)(unsigned)cb * BYTES;
 }
+// Read-only-path load: for what nothing writes while the grid is resident, links, clover and
+// tables. A programmatic dependent (launch_pdl) is resident while its predecessor still
+// writes, and its wait orders plain loads only, so fields (spinors, activations, gradients)
+// are read with ld_field. Links and clover are settled before any dependent comes up
+// (launch_settle).
 template <typename V> __device__ __forceinline__ V ldg_chunk(const char* p) {
   return __ldg(reinterpret_cast<const V*>(p));
 }
-// Read-only-cache load (NC) for fields no thread writes during the kernel, plain
-// coherent load otherwise (BLAS kernels update fields in place).
+template <typename V> __device__ __forceinline__ V ld_field(const char* p) {
+  return *reinterpret_cast<const V*>(p);
+}
+// links and clover: NC from global memory, plain from their copy in shared memory
 template <typename V, bool NC> __device__ __forceinline__ V ld_chunk(const char* p) {
-  if constexpr (NC) return __ldg(reinterpret_cast<const V*>(p));
-  else return *reinterpret_cast<const V*>(p);
+  if constexpr (NC) return ldg_chunk<V>(p);
+  else return ld_field<V>(p);
 }
 
 __device__ __forceinline__ void unpack_half8(int4 q, float v[8]) {
@@ -240,11 +247,10 @@ template <int PREC, int NR> struct SpinorIO;
 
 template <int NR> struct SpinorIO<P64, NR> {
   __host__ __device__ static constexpr size_t half_bytes(int64_t Vh) { return (size_t)NR * 8 * Vh; }
-  template <bool NC = true>
   __device__ static void load(const char* b, int Vh, int cb, double v[NR]) {
 #pragma unroll
     for (int k = 0; k < NR / 2; ++k) {
-      double2 q = ld_chunk<double2, NC>(chunk_at<16>(b, k, Vh, cb));
+      double2 q = ld_field<double2>(chunk_at<16>(b, k, Vh, cb));
       v[2 * k] = q.x; v[2 * k + 1] = q.y;
     }
   }
@@ -257,11 +263,10 @@ template <int NR> struct SpinorIO<P64, NR> {
 
 template <> struct SpinorIO<P32, 24> {
   __host__ __device__ static constexpr size_t half_bytes(int64_t Vh) { return (size_t)96 * Vh; }
-  template <bool NC = true>
   __device__ static void load(const char* b, int Vh, int cb, float v[24]) {
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-      float4 q = ld_chunk<float4, NC>(chunk_at<16>(b, k, Vh, cb));
+      float4 q = ld_field<float4>(chunk_at<16>(b, k, Vh, cb));
       v[4 * k] = q.x; v[4 * k + 1] = q.y; v[4 * k + 2] = q.z; v[4 * k + 3] = q.w;
     }
   }
@@ -275,11 +280,10 @@ template <> struct SpinorIO<P32, 24> {
 
 template <> struct SpinorIO<P32, 6> {
   __host__ __device__ static constexpr size_t half_bytes(int64_t Vh) { return (size_t)24 * Vh; }
-  template <bool NC = true>
   __device__ static void load(const char* b, int Vh, int cb, float v[6]) {
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      float2 q = ld_chunk<float2, NC>(chunk_at<8>(b, k, Vh, cb));
+      float2 q = ld_field<float2>(chunk_at<8>(b, k, Vh, cb));
       v[2 * k] = q.x; v[2 * k + 1] = q.y;
     }
   }
@@ -300,19 +304,17 @@ __device__ __forceinline__ float site_norm_scale(const float* v, int n, float& i
 template <> struct SpinorIO<P16, 24> {
   __host__ __device__ static constexpr size_t half_bytes(int64_t Vh) { return (size_t)52 * Vh; }
   // the 24 stored values without the per-site norm, which is returned
-  template <bool NC = true>
   __device__ static float load_raw(const char* b, int Vh, int cb, float v[24]) {
-    const float n = ld_chunk<float, NC>(b + (size_t)48 * Vh + (size_t)cb * 4);
+    const float n = ld_field<float>(b + (size_t)48 * Vh + (size_t)cb * 4);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) unpack_half8(ld_chunk<int4, NC>(chunk_at<16>(b, k, Vh, cb)), v + 8 * k);
+    for (int k = 0; k < 3; ++k) unpack_half8(ld_field<int4>(chunk_at<16>(b, k, Vh, cb)), v + 8 * k);
     return n;
   }
-  template <bool NC = true>
   __device__ static void load(const char* b, int Vh, int cb, float v[24]) {
-    float n = ld_chunk<float, NC>(b + (size_t)48 * Vh + (size_t)cb * 4);
+    float n = ld_field<float>(b + (size_t)48 * Vh + (size_t)cb * 4);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      int4 q = ld_chunk<int4, NC>(chunk_at<16>(b, k, Vh, cb));
+      int4 q = ld_field<int4>(chunk_at<16>(b, k, Vh, cb));
       unpack_half8(q, v + 8 * k);
     }
 #pragma unroll
@@ -333,22 +335,20 @@ template <> struct SpinorIO<P16, 24> {
 template <> struct SpinorIO<P16, 6> {
   __host__ __device__ static constexpr size_t half_bytes(int64_t Vh) { return (size_t)16 * Vh; }
   // the 6 stored values without the per-site norm, which is returned
-  template <bool NC = true>
   __device__ static float load_raw(const char* b, int Vh, int cb, float v[6]) {
-    const float n = ld_chunk<float, NC>(b + (size_t)12 * Vh + (size_t)cb * 4);
+    const float n = ld_field<float>(b + (size_t)12 * Vh + (size_t)cb * 4);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const float2 q = __half22float2(ld_chunk<__half2, NC>(chunk_at<4>(b, k, Vh, cb)));
+      const float2 q = __half22float2(ld_field<__half2>(chunk_at<4>(b, k, Vh, cb)));
       v[2 * k] = q.x; v[2 * k + 1] = q.y;
     }
     return n;
   }
-  template <bool NC = true>
   __device__ static void load(const char* b, int Vh, int cb, float v[6]) {
-    float n = ld_chunk<float, NC>(b + (size_t)12 * Vh + (size_t)cb * 4);
+    float n = ld_field<float>(b + (size_t)12 * Vh + (size_t)cb * 4);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      __half2 q = ld_chunk<__half2, NC>(chunk_at<4>(b, k, Vh, cb));
+      __half2 q = ld_field<__half2>(chunk_at<4>(b, k, Vh, cb));
       float2 f = __half22float2(q);
       v[2 * k] = f.x * n; v[2 * k + 1] = f.y * n;
     }

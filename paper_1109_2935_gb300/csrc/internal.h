@@ -56,6 +56,9 @@ void launch_export_spinor(int prec, int nr, double* dst, int parity, const char*
                           cudaStream_t st);
 void launch_pack_links(int prec, int recon, char* dst, const double* src, const Geom& g,
                        cudaStream_t st);
+// ends the writing of links and clover on the stream (kernels that follow read them through
+// the read-only path)
+void launch_settle(cudaStream_t st);
 // natural FP64 array in host memory the GPU can access <-> device layout, coalesced over
 // the host link (FP64 / FP32 storage; returns false for FP16, which uses a staging copy)
 bool launch_host_spinor(bool import, int prec, int nr, char* dev, int parity, double* nat, const Geom& g,

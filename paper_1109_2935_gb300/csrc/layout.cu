@@ -228,4 +228,11 @@ void launch_pack_links(int prec, int recon, char* dst, const double* src, const 
   else pack_links_prec<P16>(recon, dst, src, g, st);
 }
 
+// An empty kernel, launched plainly: it starts when everything before it on the stream is
+// complete and visible. A programmatic dependent behind the kernels that write links and
+// clover could come up as soon as their blocks have left; behind this one it finds data
+// that nothing writes any more, which is what its read-only-path loads ask for.
+__global__ void settle_kernel() {}
+void launch_settle(cudaStream_t st) { settle_kernel<<<1, 32, 0, st>>>(); }
+
 }  // namespace dirac

@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(TcWarps<CIN>::THREADS, 1) ptc_tc_layer_kernel(
 #pragma unroll
           for (int cc = 0; cc < CPT; ++cc) {
             float v[24];
-            SpinorIO<P32, 24>::template load<false>(buf + cc * 6 * TC_M * TPS * 16, TC_M * TPS, q, v);
+            SpinorIO<P32, 24>::load(buf + cc * 6 * TC_M * TPS * 16, TC_M * TPS, q, v);
 #pragma unroll
             for (int s2 = 0; s2 < 4; ++s2) {
               C<float> f[3];

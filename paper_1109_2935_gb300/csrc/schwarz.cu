@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(kMaxBlockSites, (SchwarzLayout<PREC, R>::kMinB
           const int lt = nbr[2 * mu + dir];
           if (lt < 0) continue;  // Dirichlet: the hop leaves the block
           T psi[24];
-          SpinorIO<RP, 24>::template load<false>(r_s, nbs, lt, psi);
+          SpinorIO<RP, 24>::load(r_s, nbs, lt, psi);
           Link<T> U;
           const int ls = dir == 0 ? t : lt;  // forward: own link; backward: the neighbour's
           if constexpr (L::kStage) {
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(kMaxBlockSites, (SchwarzLayout<PREC, R>::kMinB
         for (int k = 0; k < 6; ++k) acc[2 * blk + k / 3][k % 3] = out6[k];
       }
       T rv[24];
-      SpinorIO<RP, 24>::template load<false>(r_s, nbs, t, rv);
+      SpinorIO<RP, 24>::load(r_s, nbs, t, rv);
 #pragma unroll
       for (int s = 0; s < 4; ++s)
 #pragma unroll
@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(kMaxBlockSites, (SchwarzLayout<PREC, R>::kMinB
     }
     if (active) {
       T rv[24];
-      SpinorIO<RP, 24>::template load<false>(r_s, nbs, t, rv);
+      SpinorIO<RP, 24>::load(r_s, nbs, t, rv);
 #pragma unroll
       for (int k = 0; k < 12; ++k) {
         T rr = rv[2 * k], ri = rv[2 * k + 1];

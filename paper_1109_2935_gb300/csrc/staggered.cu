@@ -116,8 +116,8 @@ __device__ __forceinline__ void stag_mv_h(const uint32_t* uw, const uint32_t chi
 // a 16-bit colour vector (3 binary16 words) and its norm
 __device__ __forceinline__ float load_stag_h(const char* src, int Vh, int cb, uint32_t chi[3]) {
 #pragma unroll
-  for (int k = 0; k < 3; ++k) chi[k] = __ldg(reinterpret_cast<const uint32_t*>(src + ((size_t)k * Vh + cb) * 4));
-  return __ldg(reinterpret_cast<const float*>(src + (size_t)12 * Vh) + cb);
+  for (int k = 0; k < 3; ++k) chi[k] = ld_field<uint32_t>(chunk_at<4>(src, k, Vh, cb));
+  return ld_field<float>(chunk_at<4>(src, 3, Vh, cb));
 }
 // the stored words of a 16-bit link with R = 18 (9 words) or 12 (6 words) reals
 template <int R>

@@ -237,11 +237,11 @@ __device__ __forceinline__ void herm6_hh(const uint32_t blk[18], const uint32_t 
 // the site's own spinor; their two per-site norms scale the 12 results once.
 __device__ __forceinline__ void clover_self_h(const char* clov, const char* self, int Vh, int cb, C<float> av[12]) {
   const float nc = __ldg(reinterpret_cast<const float*>(clov + (size_t)144 * Vh) + cb);
-  const float ns = __ldg(reinterpret_cast<const float*>(self + (size_t)48 * Vh) + cb);
+  const float ns = ld_field<float>(chunk_at<4>(self, 12, Vh, cb));
   uint32_t x[12];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const int4 q = ldg_chunk<int4>(chunk_at<16>(self, k, Vh, cb));
+    const int4 q = ld_field<int4>(chunk_at<16>(self, k, Vh, cb));
     x[4 * k] = (uint32_t)q.x; x[4 * k + 1] = (uint32_t)q.y; x[4 * k + 2] = (uint32_t)q.z; x[4 * k + 3] = (uint32_t)q.w;
   }
   // block 0: words 0..17 (chunks 0..3 and half of chunk 4); block 1: words 18..35
@@ -269,13 +269,12 @@ __device__ __forceinline__ void clover_self_h(const char* clov, const char* self
 // A 16-bit neighbour spinor for a hop: the upper two spin components converted (u, 12
 // reals), the lower two kept as binary16 pairs (l, 6 words: spin 2 colours 0..2, spin 3
 // colours 0..2, re low / im high); returns bc times the site norm, the hop's factor.
-template <bool NC = true>
 __device__ __forceinline__ float load_hop_h(const char* src, int Vh, int cb, float u[12], uint32_t l[6], float bc) {
-  const float n = ld_chunk<float, NC>(chunk_at<4>(src, 12, Vh, cb));
+  const float n = ld_field<float>(chunk_at<4>(src, 12, Vh, cb));
   uint32_t w[12];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const int4 q = ld_chunk<int4, NC>(chunk_at<16>(src, k, Vh, cb));
+    const int4 q = ld_field<int4>(chunk_at<16>(src, k, Vh, cb));
     w[4 * k] = (uint32_t)q.x; w[4 * k + 1] = (uint32_t)q.y; w[4 * k + 2] = (uint32_t)q.z; w[4 * k + 3] = (uint32_t)q.w;
   }
 #pragma unroll
@@ -367,10 +366,10 @@ __device__ __forceinline__ void clover_site_n(const char* clov, const char* self
         uint32_t x[8];
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
-          const int4 q = ldg_chunk<int4>(chunk_at<16>(s, blk + k, Vh, cb));
+          const int4 q = ld_field<int4>(chunk_at<16>(s, blk + k, Vh, cb));
           x[4 * k] = (uint32_t)q.x; x[4 * k + 1] = (uint32_t)q.y; x[4 * k + 2] = (uint32_t)q.z; x[4 * k + 3] = (uint32_t)q.w;
         }
-        const float n = nc * __ldg(reinterpret_cast<const float*>(chunk_at<4>(s, 12, Vh, cb)));
+        const float n = nc * ld_field<float>(chunk_at<4>(s, 12, Vh, cb));
         C<float> y[6];
         herm6_hh(c + 2 * blk, x + 2 * blk, y);
 #pragma unroll
@@ -391,7 +390,7 @@ __device__ __forceinline__ void clover_site_n(const char* clov, const char* self
         C<float> x[6], y[6];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          const float4 q = ldg_chunk<float4>(chunk_at<16>(self + r * stride, 3 * blk + k, Vh, cb));
+          const float4 q = ld_field<float4>(chunk_at<16>(self + r * stride, 3 * blk + k, Vh, cb));
           x[2 * k] = C<float>{q.x, q.y};
           x[2 * k + 1] = C<float>{q.z, q.w};
         }
@@ -477,7 +476,7 @@ __device__ __forceinline__ void ring_hop(C<float> acc[N][4][3], const char* slot
   for (int r = 0; r < N; ++r) {
     float u[12];
     uint32_t l[6];
-    const float n = load_hop_h<false>(slot + r * 52 * T, T, t, u, l, bc);
+    const float n = load_hop_h(slot + r * 52 * T, T, t, u, l, bc);
     wilson_hop_h<MU>(acc[r], u, l, U, dag, s, n);
   }
 }

@@ -11,11 +11,10 @@ namespace dirac {
 template <> struct Real<P64DS> { using T = dsf; };
 
 template <> struct SpinorIO<P64DS, 24> {
-  template <bool NC = true>
   __device__ static void load(const char* b, int Vh, int cb, dsf v[24]) {
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-      const double2 q = ld_chunk<double2, NC>(b + ((size_t)k * Vh + cb) * 16);
+      const double2 q = ld_field<double2>(b + ((size_t)k * Vh + cb) * 16);
       v[2 * k] = dsf(q.x);
       v[2 * k + 1] = dsf(q.y);
     }

@@ -84,8 +84,8 @@ __global__ void __launch_bounds__(32) wilson_split64_kernel(const WilsonArg a) {
     double2 u[3], w[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      u[c] = ldg_chunk<double2>(src + ((size_t)(3 * spin + c) * Vh + ycb) * 16);
-      w[c] = ldg_chunk<double2>(src + ((size_t)(6 + 3 * low + c) * Vh + ycb) * 16);
+      u[c] = ld_field<double2>(src + ((size_t)(3 * spin + c) * Vh + ycb) * 16);
+      w[c] = ld_field<double2>(src + ((size_t)(6 + 3 * low + c) * Vh + ycb) * 16);
     }
     Link<double> U, W;
     LinkIO<P64, R>::load(a.gauge, Vh, mu, back ? 1 - par : par, back ? ycb : cb, U);
@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(32) wilson_split64_kernel(const WilsonArg a) {
   const char* self = FULLM ? (par ? a.in[1] : a.in[0]) : a.self;
   const char* cself = FULLM ? a.clover : a.c_self;
   C<double> acc = {0, 0}, av = {0, 0}, out;
-  auto self_at = [&](int e) { return ldg_chunk<double2>(self + ((size_t)e * Vh + cb) * 16); };
+  auto self_at = [&](int e) { return ld_field<double2>(self + ((size_t)e * Vh + cb) * 16); };
   if (self) {
     if (cself) {
       av = row64(cself + par * pb, Vh, cb, k >= 6, k >= 6 ? k - 6 : k, self_at);
