@@ -15,15 +15,18 @@
 namespace dirac {
 
 // Launches that follow one another on a stream (the steps of a solver, the hops of an
-// even-odd operator) start without the gap between two kernels: launch_pdl lets a grid
-// become resident while its predecessor runs, and pdl_begin, the first statement of every
-// kernel launched this way, waits until that predecessor is complete and its writes are
-// visible, then lets the successor come up. Without the attribute both are no-ops, and any
-// other work on the stream is ordered as ever.
-__device__ __forceinline__ void pdl_begin() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
+// even-odd operator) start without the gap between two kernels: launch_pdl lets a grid come
+// up as soon as every block of its predecessor has left, before the predecessor counts as
+// complete, and pdl_begin, the first statement of every kernel launched this way, waits for
+// that completion and its writes. Without the attribute it is a no-op, and any other work on
+// the stream is ordered as ever. No kernel lets its successor come up earlier
+// (griddepcontrol.launch_dependents): blocks that become resident beside a running grid take
+// the slots that it happens to leave, so a grid of a few blocks per SM ends up uneven, and
+// one bound by the FP64 pipes runs as long as its fullest SM. With that instruction, against
+// the form here (us per iteration): asqtad CG FP64 16^4 403 -> 223 (252 without dependent
+// launches), FP32 16^3x32 97 -> 72; BiCGstab FP64 8^4 124 -> 89; even-odd 12^3x16 392 -> 275;
+// CG FP64 4^4 32.4 -> 32.0 (46 without).
+__device__ __forceinline__ void pdl_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <class... P, class... A>
 inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchAttribute at{};
@@ -209,9 +212,9 @@ template <int BYTES> __device__ __forceinline__ const char* chunk_at(const char*
   return b + (size_t)k * Vh * BYTES + (size_t)(unsigned)cb * BYTES;
 }
 // Read-only-path load: for what nothing writes while the grid is resident, links, clover and
-// tables. A programmatic dependent (launch_pdl) is resident while its predecessor still
-// writes, and its wait orders plain loads only, so fields (spinors, activations, gradients)
-// are read with ld_field. Links and clover are settled before any dependent comes up
+// tables. A programmatic dependent (launch_pdl) may be resident before its predecessor's
+// writes are complete, and its wait orders plain loads only, so fields (spinors, activations,
+// gradients) are read with ld_field. Links and clover are settled before any dependent comes up
 // (launch_settle).
 template <typename V> __device__ __forceinline__ V ldg_chunk(const char* p) {
   return __ldg(reinterpret_cast<const V*>(p));

@@ -1,5 +1,5 @@
-"""Kernels launched as programmatic dependents are resident while their predecessor still
-writes. So each begins with the wait, and reads through the read-only path (__ldg: data that
+"""Kernels launched as programmatic dependents may be resident before their predecessor is
+complete. So each begins with the wait, and reads through the read-only path (__ldg: data that
 nothing writes during the kernel) only links, clover and tables, never a field that the
 predecessor may have produced. Checked on the source text."""
 import os
@@ -80,3 +80,10 @@ def test_links_and_clover_are_settled_before_a_dependent():
     assert last_write < load.index("launch_settle(st)") < load.index("have_gauge = true")
     for f, s in _sources().items():  # and launched plainly: it waits for the writers' completion
         assert not re.search(r"launch_pdl\(settle_kernel", s), f
+
+
+def test_no_kernel_lets_its_successor_come_up_beside_it():
+    """Blocks that become resident beside a running grid are placed unevenly, which doubles the
+    time of grids of a few blocks per SM: successors come up when the blocks have left."""
+    for f, s in _sources().items():
+        assert "launch_dependents" not in s, f
