@@ -748,17 +748,21 @@ static int run_reduce(Blas* b, const Op& op, int n, double* out, int nout, cudaS
 }
 
 // Storage of an operation's fields: 0 no FP64, 1 FP64 and others (FP64 arithmetic), 2 FP64
-// only: chunk by chunk (NR = 2; a thread per site would issue 12 x the FP64 instructions in
-// a row, each 64 cycles: CG update on 4^4 20.7 us).
+// only and few sites: chunk by chunk (NR = 2; a thread per site would issue 12 x the FP64
+// instructions in a row, each 64 cycles: CG update on 4^4 20.7 us). On more sites a thread
+// per site fills the chip, and its loads in flight are what counts. Measured, whole call, us,
+// site -> chunk: (x, y) and ||x||^2 at 8,192 sites 29.6 -> 27.5, 16,384 29.2 -> 29.8, 27,648
+// 29.2 -> 32.0, 884,736 142 -> 207; per iteration of GCR at 13,824 sites (even-odd) 182 -> 172,
+// at 27,648 196 -> 208.
 enum : int { NO64 = 0, SOME64 = 1, ALL64 = 2 };
+constexpr int kChunkSites = 16384;
 static int kind(std::initializer_list<const FieldRef*> fs) {
   bool all = true, some = false;
   for (auto f : fs) {
     all = all && f->prec == P64;
     some = some || f->prec == P64;
   }
-  const FieldRef& f = **fs.begin();
-  all = all && (int64_t)nsites(f) * (f.nr / 2) < ((int64_t)1 << 30);  // NS is an int
+  all = all && nsites(**fs.begin()) <= kChunkSites;
   return all ? ALL64 : some ? SOME64 : NO64;
 }
 
