@@ -10,6 +10,8 @@
 // plan can record its launches in a CUDA graph for replay. With FP16 storage the plan
 // also times the tensor-core kernel of mrhs_tc.cu (all right-hand sides of a site in
 // one dense contraction) and keeps the faster of the two.
+#include <algorithm>
+#include <climits>
 #include <cmath>
 #include <string>
 #include <vector>
@@ -109,12 +111,14 @@ __global__ void __launch_bounds__(kTileSites * kMaxRG, 1)
   }
 }
 
-// FP64 fields: a warp per (right-hand side, 32-site group), over the right-hand sides that
-// the masks leave. The FP64 pipe bounds this kernel (19 cycles per warp instruction and SM,
+// FP64 fields of a masked plan (the FP64 residuals of the batched solves): a warp per
+// (right-hand side, 32-site group), over the right-hand sides that the masks leave. The FP64 pipe bounds this kernel (19 cycles per warp instruction and SM,
 // four schedulers at 64), links and clover come from L2 at a tenth of its rate, so what
 // counts is that every scheduler has the same number of warps with work: with warp y of a
 // CTA tied to right-hand side 4 k + y, a reliable update of a few systems ran on one or two
-// of the four schedulers.
+// of the four schedulers. Without a mask the tuned shapes of batch_kernel are faster (us, that
+// -> this): 8^3x16 x 1 43 -> 73, 12^3x20 x 1 80 -> 117, 10^2x14x18 x 3 158 -> 193, 16^4 x 3
+// 408 -> 423.
 static constexpr int kBatch64PerSM = 3;
 static constexpr int kMaxBatch64Rhs = 1024;  // right-hand sides listed at a time
 template <int R>
@@ -257,6 +261,7 @@ struct dirac_batch {
   int prec = 0, recon = 12, ntiles = 0, nrhs = 0;
   bool ds = false;               // FP64 fields: double-single arithmetic (18-real links)
   int RG = 1, NR = 1, per_sm = 1, grid = 1;
+  int grid64 = 1;                // CTAs of the kernel for masked FP64 plans
   double tuned_ms = 0;
   std::vector<double> cand_ms;   // autotuner timings, candidate order
   cudaGraph_t graph = nullptr;
@@ -329,7 +334,8 @@ static void batch_launch_direct(dirac_batch* b, cudaStream_t st) {
   }
   if (b->prec == P64 && b->ds)
     launch_pdl(batch_kernel_ds, b->grid, dim3(kTileSites, 4), 0, st, b->d_lats, nlat, b->ntiles);
-  else if (b->prec == P64) launch_batch64(b->recon, b->d_lats, nlat, b->nrhs, b->grid, st);
+  else if (b->prec == P64 && b->lats[0].mask) launch_batch64(b->recon, b->d_lats, nlat, b->nrhs, b->grid64, st);
+  else if (b->prec == P64) launch_batch_prec<P64, 1>(b->recon, b->lats, b->ntiles, b->RG, b->grid, st);
   else if (b->prec == P32) (b->NR == 2 ? launch_batch_prec<P32, 2> : launch_batch_prec<P32, 1>)(b->recon, b->lats, b->ntiles, b->RG, b->grid, st);
   else (b->NR == 2 ? launch_batch_prec<P16, 2> : launch_batch_prec<P16, 1>)(b->recon, b->lats, b->ntiles, b->RG, b->grid, st);
 }
@@ -395,8 +401,9 @@ int batch_create(dirac_ctx* const* ctxs, int nlat, void* const* out, const void*
     r0 += nrhs[l];
     b->nrhs = r0;
   }
-  // FP64 fields have one kernel and one shape (batch_kernel64)
-  const bool k64 = prec == P64 && !ds;
+  long ctas64 = 0;
+  for (const BatchLat& L : b->lats) ctas64 += (long)L.tiles_site * ((L.nrhs + 3) / 4);
+  b->grid64 = grid_for(kBatch64PerSM, (int)std::min(ctas64, (long)INT_MAX));
   if (cudaMalloc(&b->d_lats, sizeof(BatchLat) * nlat) != cudaSuccess) {
     cudaGetLastError();
     delete b;
@@ -422,7 +429,7 @@ int batch_create(dirac_ctx* const* ctxs, int nlat, void* const* out, const void*
     b->NR = kCand[k][2];
     // tune < 2: only the default shape (4 right-hand sides per CTA)
     // (the default shape also serves plans with fewer right-hand sides: idle warps exit)
-    if (tune < 2 || k64 ? k != untimed : (RG > max_rhs && RG > 1) || (kCand[k][2] == 2) != pairs) {
+    if (tune < 2 ? k != untimed : (RG > max_rhs && RG > 1) || (kCand[k][2] == 2) != pairs) {
       b->cand_ms.push_back(-1);
       continue;
     }
@@ -434,7 +441,7 @@ int batch_create(dirac_ctx* const* ctxs, int nlat, void* const* out, const void*
     }
     b->RG = RG;
     if (batch_layout(b, RG, st)) break;
-    b->grid = grid_for(k64 ? kBatch64PerSM : per_sm, b->ntiles);
+    b->grid = grid_for(per_sm, b->ntiles);
     batch_launch_direct(b, st);
     cudaEventRecord(e0, st);
     for (int r = 0; r < 3; ++r) batch_launch_direct(b, st);
@@ -458,7 +465,7 @@ int batch_create(dirac_ctx* const* ctxs, int nlat, void* const* out, const void*
   }
   b->RG = kCand[bi][0];
   b->NR = kCand[bi][2];
-  b->per_sm = k64 ? kBatch64PerSM : kCand[bi][1];
+  b->per_sm = kCand[bi][1];
   if (batch_layout(b, b->RG, st)) {
     cudaFree(b->d_lats);
     delete b;
