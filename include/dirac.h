@@ -168,6 +168,12 @@ int dirac_batch_capture(dirac_batch* plan, int napply, void* stream);
 int dirac_batch_info(const dirac_batch* plan, int* rhs_per_cta, int* ctas_per_sm, int* grid,
                      double* tuned_ms);
 int dirac_batch_destroy(dirac_batch* plan);
+/* Right-hand sides per thread of the CUDA-core kernel (1 or 2; FP64 plans: 1): the plan
+ * times both and keeps the faster. set: that form in its default shape instead, on the
+ * CUDA-core kernel; a captured graph is dropped. The results are the same bytes. Returns
+ * DIRAC_ERR_UNSUPPORTED for 2 with FP64 storage. */
+int dirac_batch_rhs_per_thread(const dirac_batch* plan);
+int dirac_batch_set_rhs_per_thread(dirac_batch* plan, int n, void* stream);
 /* Tensor-core form of the batched operator, for FP16 storage with 12- or 18-real links
  * (not in the paper: a multi-right-hand-side extension). Per site the link-times-
  * spinor products of all right-hand sides of a tile are one dense contraction (Eq. 2:

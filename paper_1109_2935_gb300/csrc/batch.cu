@@ -278,10 +278,11 @@ struct dirac_batch {
 
 namespace dirac {
 
-// the tile-shape candidates: (right-hand sides per CTA, resident CTAs per SM, right-hand
-// sides per thread); all fill the 16 warps per SM of the 128-register cap
-static const int kCand[][3] = {{1, 16, 1}, {2, 8, 1}, {4, 4, 1}, {8, 2, 1}, {2, 16, 2}, {4, 8, 2}, {8, 4, 2}};
-static constexpr int kDefaultCand = 2, kDefaultPair = 5;
+// the tile-shape candidates: (right-hand sides per CTA, CTAs per SM, right-hand sides per
+// thread). 16 warps of the 128-register cap are resident per SM; the shapes with 32 hand the
+// CTAs that do not fit to the SMs that finish first, which evens out ragged ends.
+static const int kCand[][3] = {{1, 16, 1}, {2, 8, 1}, {4, 4, 1}, {2, 16, 1}, {4, 8, 1}, {2, 16, 2}, {4, 8, 2}, {8, 4, 2}};
+static constexpr int kDefaultCand = 2, kDefaultPair = 6;
 
 // Two right-hand sides per thread load and rebuild every link once for both, but a thread
 // takes about 1.6 times as long and there are half as many: worth it from about two waves of
@@ -410,7 +411,11 @@ int batch_create(dirac_ctx* const* ctxs, int nlat, void* const* out, const void*
     return DIRAC_ERR_OOM;
   }
   // autotune: time every candidate shape once (after one warm-up launch) and keep the
-  // fastest; the launches write the plan's outputs, which the caller owns anyway
+  // fastest; the launches write the plan's outputs, which the caller owns anyway. One and two
+  // right-hand sides per thread are both timed: which is faster turns on whether links and
+  // clover come from L2 (FP16 12^3x20 x 8 24.7 us against 26.5, 10^2x14x18 x 10 22.5 against
+  // 25.4) or from DRAM (FP32 24^3x32 x 9 409 against 354), and lattices of both kinds may share
+  // a plan.
   cudaStream_t st = stream;
   int max_rhs = 1;
   for (int l = 0; l < nlat; ++l) max_rhs = nrhs[l] > max_rhs ? nrhs[l] : max_rhs;
@@ -429,7 +434,7 @@ int batch_create(dirac_ctx* const* ctxs, int nlat, void* const* out, const void*
     b->NR = kCand[k][2];
     // tune < 2: only the default shape (4 right-hand sides per CTA)
     // (the default shape also serves plans with fewer right-hand sides: idle warps exit)
-    if (tune < 2 ? k != untimed : (RG > max_rhs && RG > 1) || (kCand[k][2] == 2) != pairs) {
+    if (tune < 2 ? k != untimed : (RG > max_rhs && RG > 1) || (prec == P64 && b->NR > 1)) {
       b->cand_ms.push_back(-1);
       continue;
     }
@@ -443,17 +448,20 @@ int batch_create(dirac_ctx* const* ctxs, int nlat, void* const* out, const void*
     if (batch_layout(b, RG, st)) break;
     b->grid = grid_for(per_sm, b->ntiles);
     batch_launch_direct(b, st);
-    cudaEventRecord(e0, st);
-    for (int r = 0; r < 3; ++r) batch_launch_direct(b, st);
-    cudaEventRecord(e1, st);
-    if (cudaEventSynchronize(e1) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
-      b->err = "autotune launch failed";
-      break;
-    }
+    // one launch, or the mean of three where one is short
     float ms = 0;
-    cudaEventElapsedTime(&ms, e0, e1);
-    b->cand_ms.push_back(ms / 3);
-    if (ms / 3 < best) { best = ms / 3; bi = k; }
+    for (int reps = 1; reps <= 3 && b->err.empty(); reps += 2) {
+      cudaEventRecord(e0, st);
+      for (int r = 0; r < reps; ++r) batch_launch_direct(b, st);
+      cudaEventRecord(e1, st);
+      if (cudaEventSynchronize(e1) != cudaSuccess || cudaGetLastError() != cudaSuccess) b->err = "autotune launch failed";
+      cudaEventElapsedTime(&ms, e0, e1);
+      ms /= reps;
+      if (ms > 0.5f) break;
+    }
+    if (!b->err.empty()) break;
+    b->cand_ms.push_back(ms);
+    if (ms < best) { best = ms; bi = k; }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -625,6 +633,24 @@ int dirac_batch_set_tensor_cores(dirac_batch* b, int on) {
   }
   b->use_tc = on != 0;
   b->tuned_ms = b->use_tc ? b->tc_ms : b->cc_ms;
+  return DIRAC_OK;
+}
+
+int dirac_batch_rhs_per_thread(const dirac_batch* b) { return b ? b->NR : 0; }
+
+int dirac_batch_set_rhs_per_thread(dirac_batch* b, int n, void* stream) {
+  if (!b || n < 1 || n > 2) return DIRAC_ERR_ARG;
+  if (n == 2 && b->prec == P64) return DIRAC_ERR_UNSUPPORTED;
+  if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
+  if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
+  b->graph_napply = 0;
+  const int* shape = kCand[n == 2 ? kDefaultPair : kDefaultCand];
+  b->use_tc = false;
+  b->RG = shape[0];
+  b->per_sm = shape[1];
+  b->NR = n;
+  if (batch_layout(b, b->RG, (cudaStream_t)stream)) return DIRAC_ERR_CUDA;
+  b->grid = grid_for(b->per_sm, b->ntiles);
   return DIRAC_OK;
 }
 

@@ -97,6 +97,8 @@ _SIGS = {
     "dirac_batch_info": (_ci, [_vp, ctypes.POINTER(_ci), ctypes.POINTER(_ci), ctypes.POINTER(_ci),
                                ctypes.POINTER(ctypes.c_double)]),
     "dirac_batch_destroy": (_ci, [_vp]),
+    "dirac_batch_rhs_per_thread": (_ci, [_vp]),
+    "dirac_batch_set_rhs_per_thread": (_ci, [_vp, _ci, _vp]),
     "dirac_batch_set_tensor_cores": (_ci, [_vp, _ci]),
     "dirac_batch_kernel_info": (_ci, [_vp, ctypes.POINTER(_ci), _pd, _pd]),
     "dirac_norm2": (_ci, [_vp, _vp, _ci, _ci, _pd, _vp]),
@@ -373,7 +375,13 @@ class Batch:
         rg, per, grid, ms = _ci(), _ci(), _ci(), ctypes.c_double()
         dirac_batch_info(self.plan, ctypes.byref(rg), ctypes.byref(per), ctypes.byref(grid), ctypes.byref(ms))
         return {"rhs_per_cta": rg.value, "ctas_per_sm": per.value, "grid": grid.value,
-                "tuned_ms": ms.value}
+                "tuned_ms": ms.value, "rhs_per_thread": dirac_batch_rhs_per_thread(self.plan)}
+
+    def set_rhs_per_thread(self, n, stream=None):
+        """The CUDA-core kernel with n (1 or 2) right-hand sides per thread, in its default shape."""
+        rc = dirac_batch_set_rhs_per_thread(self.plan, n, _stream(stream))
+        if rc != OK:
+            raise DiracError(rc, "dirac_batch_set_rhs_per_thread failed")
 
     def set_tensor_cores(self, on):
         """Select the tensor-core kernel (FP16 storage) or the CUDA-core kernel."""
