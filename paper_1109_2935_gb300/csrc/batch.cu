@@ -98,12 +98,12 @@ __global__ void __launch_bounds__(kTileSites * kMaxRG, 1) mrhs_kernel(const __gr
 }
 
 // several lattices: descriptor table in the parameter space (uniform loads), tiles numbered
-// across lattices. Launched plainly: as a programmatic dependent of its own predecessor the
-// grid of resident CTAs took 3.13 instead of 2.99 ms (3 lattices x 12, FP16).
+// across lattices
 struct LatTable { BatchLat v[kMaxLat]; };
 template <int PREC, int R, int NR>
 __global__ void __launch_bounds__(kTileSites * kMaxRG, 1)
     batch_kernel(const __grid_constant__ LatTable lats, int nlat, int ntiles, int RG) {
+  pdl_begin();
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
     int l = 0;
     while (l + 1 < nlat && t >= lats.v[l + 1].tile_begin) ++l;
@@ -203,9 +203,9 @@ static void launch_batch_prec(int recon, const std::vector<BatchLat>& l, int nti
   for (size_t k = 0; k < l.size(); ++k) t.v[k] = l[k];
   const int nlat = (int)l.size();
   dim3 block(kTileSites, RG / NR);
-  if (recon == 18) batch_kernel<PREC, 18, NR><<<grid, block, (RG / NR * kRingWarp<PREC, 18, NR>), st>>>(t, nlat, ntiles, RG);
-  else if (recon == 12) batch_kernel<PREC, 12, NR><<<grid, block, (RG / NR * kRingWarp<PREC, 12, NR>), st>>>(t, nlat, ntiles, RG);
-  else batch_kernel<PREC, 8, NR><<<grid, block, (RG / NR * kRingWarp<PREC, 8, NR>), st>>>(t, nlat, ntiles, RG);
+  if (recon == 18) launch_pdl(batch_kernel<PREC, 18, NR>, grid, block, RG / NR * kRingWarp<PREC, 18, NR>, st, t, nlat, ntiles, RG);
+  else if (recon == 12) launch_pdl(batch_kernel<PREC, 12, NR>, grid, block, RG / NR * kRingWarp<PREC, 12, NR>, st, t, nlat, ntiles, RG);
+  else launch_pdl(batch_kernel<PREC, 8, NR>, grid, block, RG / NR * kRingWarp<PREC, 8, NR>, st, t, nlat, ntiles, RG);
 }
 
 static void launch_batch64(int recon, const BatchLat* d, int nlat, int nrhs, int grid, cudaStream_t st) {

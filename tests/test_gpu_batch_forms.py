@@ -115,3 +115,12 @@ def test_masked_pairs_on_lattices_that_take_pairs(dirac, sloppy):
             x1 = torch.zeros(n, dtype=torch.uint8, device="cuda")
             dirac.solve_many([lat], [x1], [b[r * n:(r + 1) * n].clone()], [1], tol=1e-10, prec_sloppy=sloppy)
             assert torch.equal(x1, x[r * n:(r + 1) * n])
+
+
+@pytest.mark.parametrize("dims,nrhs", [((8, 8, 8, 16), 11), ((16, 16, 16, 16), 3)])
+def test_plan_launches_follow_as_closely_as_unplanned_ones(dirac, dims, nrhs):
+    """Both are dependent launches of the same stencil; a plain one would add 2 us to 9."""
+    import torch
+    lat, x, _, plan = _plan(dirac, dims, F32, nrhs)
+    z = torch.zeros_like(x)
+    assert best_us(plan.apply) < 1.1 * best_us(lambda: lat.apply_multi(z, x, nrhs, F32))
