@@ -286,14 +286,17 @@ static constexpr int kDefaultCand = 2, kDefaultPair = 6;
 
 // Two right-hand sides per thread load and rebuild every link once for both, but a thread
 // takes about 1.6 times as long and there are half as many: worth it from about two waves of
-// resident warps on (16 per SM). Measured, one right-hand side per thread -> two, us: FP32
-// 12^3x20 x 7 26.8 -> 22.9, 16^4 x 12 102.6 -> 80.8, 16^3x32 x 2 33.0 -> 29.2, 8^4 x 12 8.6 ->
-// 9.1; FP16 16^4 x 12 80.2 -> 66.0, 16^3x32 x 7 84.0 -> 89.3, 12^3x20 x 12 38.6 -> 37.1, 8^3x16
-// x 7 8.8 -> 10.2. With an odd count one thread of each group has a single right-hand side,
-// which FP16 (compute-bound) does not make up for.
+// resident warps on (16 per SM), most where links and clover come from DRAM. The rule of the
+// calls that are not timed. Measured, one right-hand side per thread -> two, us: FP32 12^3x20 x
+// 7 20.9 -> 20.1, 16^4 x 12 65 -> 66, 16^3x32 x 2 29.0 -> 26.5, x 12 148 -> 127, 24^3x32 x 12
+// 510 -> 413; FP16 16^4 x 12 62.0 -> 61.3, 16^3x32 x 8 82.6 -> 76.4, 24^3x32 x 8 284 -> 252; below
+// two waves 12^3x20 x 8 FP16 21.7 -> 22.6, 8^3x16 x 7 6.8 -> 7.9. With an odd count one thread of
+// each group has a single right-hand side: FP32 still gains (16^4 x 3 18.0 -> 17.1, 24^3x32 x 3
+// 154 -> 127, x 5 252 -> 206), FP16, which is compute-bound, does not (16^3x32 x 7 73.3 -> 79.2, x
+// 15 162 -> 165).
 static bool pair_rhs(int prec, long groups, int nrhs) {
   if (prec == P64 || groups * nrhs <= 32l * sm_count()) return false;
-  return nrhs % 2 == 0 || (prec == P32 && nrhs >= 5);
+  return nrhs % 2 == 0 || (prec == P32 && nrhs >= 3);
 }
 
 // Warps per CTA for `items` warps on the same sites: the most (up to 4, they share the links
@@ -355,7 +358,12 @@ int dirac_apply_multi(dirac_ctx* c, void* out, const void* in, int nrhs, dirac_p
   const char *i0 = (const char*)in, *o0 = (const char*)out;
   if (i0 < o0 + fb * nrhs && o0 < i0 + fb * nrhs) return set_err(c, DIRAC_ERR_ARG, "in and out overlap");
   const int NR = pair_rhs(prec, full_sites((int)c->Vh) / kTileSites, nrhs) ? 2 : 1;
-  const int warps = group_warps((nrhs + NR - 1) / NR), RG = warps * NR;
+  int warps = group_warps((nrhs + NR - 1) / NR);
+  // an odd count leaves the last warp of its CTA a single right-hand side on every tile: with
+  // two warps half of the chip's work is out of step (FP32 24^3x32 x 3 148 us against 127 with
+  // one warp per CTA, 16^4 x 11 70 against 63)
+  if (NR == 2 && nrhs % 2 && warps < 4) warps = 1;
+  const int RG = warps * NR;
   const BatchLat L = describe(c, prec, in, out, nrhs, RG);
   const int grid = grid_for(16 / warps, L.tiles);
   cudaStream_t st = (cudaStream_t)stream;
