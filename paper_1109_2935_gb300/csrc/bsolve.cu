@@ -682,6 +682,7 @@ int solve_batched_impl(Run& R, const dirac_solver_params& P, dirac_solver_stats*
   if (cudaStreamSynchronize(R.st) != cudaSuccess) return DIRAC_ERR_CUDA;
   std::vector<double> target(n), rmax(n), rr(n);
   std::vector<int> active(n, 1), relup(n, 0), stale(n, 0), settled(n, 0);
+  std::vector<int> applied(n, 0);  // operator applications of each system
   for (int j = 0; j < n; ++j) R.upd_h()[j] = 1;  // the start covers every right-hand side
   for (int j = 0; j < n; ++j) {
     bb[j] = R.hgathered()[j];
@@ -695,6 +696,7 @@ int solve_batched_impl(Run& R, const dirac_solver_params& P, dirac_solver_stats*
     // r = b - M x from the caller's x; the sloppy and shadow residuals from it
     RT(launch(R, OpInit<SP, AP, true>{}));
     RT(dirac_batch_apply(R.plan_x, R.st));
+    applied.assign(n, 1);
     RT(launch(R, OpXmy{}));
     RT(launch(R, OpRestart<SP>{}));
     RT(launch(R, OpShadow<SP>{}));
@@ -751,7 +753,10 @@ int solve_batched_impl(Run& R, const dirac_solver_params& P, dirac_solver_stats*
     cudaEventRecord(ev[slot], R.st);
     ++total;
     for (int j = 0; j < n; ++j)
-      if (active[j]) stats[j].iters++;
+      if (active[j]) {
+        stats[j].iters++;
+        applied[j] += 2;
+      }
     if (it > 0) {
       // the previous iteration's residuals decide reliable updates and convergence
       const int ps = (it - 1) & 1;
@@ -785,11 +790,13 @@ int solve_batched_impl(Run& R, const dirac_solver_params& P, dirac_solver_stats*
         bool fresh = false;
         for (int j = 0; rc == DIRAC_OK && j < n; ++j)
           fresh = fresh || (R.upd_h()[j] != 0 && R.hgathered()[j] < target[j]);
-        if (rc == DIRAC_OK && fresh && R.plan_xds) rc = residual(R, R.plan_x);
+        const bool again = fresh && R.plan_xds;
+        if (rc == DIRAC_OK && again) rc = residual(R, R.plan_x);
         if (rc == DIRAC_OK) {
           for (int j = 0; j < n; ++j) {
             R.active_h()[j] = active[j];
             if (R.upd_h()[j] == 0) continue;
+            applied[j] += again ? 2 : 1;
             rr[j] = R.hgathered()[j];
             relup[j]++;
             stale[j] = 1;
@@ -819,6 +826,7 @@ int solve_batched_impl(Run& R, const dirac_solver_params& P, dirac_solver_stats*
     } else {
       for (int j = 0; j < n; ++j) {
         R.upd_h()[j] = settled[j] ? 0 : 1;
+        applied[j] += settled[j] ? 0 : 1;
         left = left || !settled[j];
       }
       if (left) rc = reliable<SP, AP>(R, true);
@@ -833,7 +841,7 @@ int solve_batched_impl(Run& R, const dirac_solver_params& P, dirac_solver_stats*
   for (int j = 0; j < n; ++j) {
     stats[j].reliable_updates = relup[j];
     stats[j].true_rel_resid = bb[j] > 0 ? std::sqrt(rr[j] / bb[j]) : 0.0;
-    stats[j].dslash_calls = 2 * stats[j].iters + relup[j] + 1;
+    stats[j].dslash_calls = applied[j];
   }
   return rc;
 }
