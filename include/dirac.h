@@ -369,7 +369,8 @@ int dirac_ptc_gradient(dirac_ptc* net, const void* r, const void* v, double* los
  * ||K r_i - v_i||^2 / ||v_i||^2. r may be NULL: then r_i = M v_i is computed (FP32)
  * by the library. r[i], v[i]: FP32 full fields owned by the caller, unchanged.
  * loss (host, may be NULL): params->steps entries, the batch loss before each step.
- * Synchronises stream. */
+ * The sources made here and the loss history stay allocated with the network for the next
+ * call, up to 256 MB and 1 MB; what is larger is freed. Synchronises stream. */
 int dirac_ptc_train(dirac_ptc* net, const void* const* r, const void* const* v, int npairs,
                     const dirac_ptc_train_params* params, double* loss, void* stream);
 /* on = 1: dirac_ptc_apply and the GCR_PTC solver run every layer on the tensor cores

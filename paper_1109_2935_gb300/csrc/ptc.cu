@@ -556,7 +556,7 @@ struct dirac_ptc {
   float* partial = nullptr;
   size_t partial_bytes = 0;
   double* dsc = nullptr;   // [0, MAXB): inv; [MAXB]: loss; then norm / loss partials
-  char* tr = nullptr;      // training: sources r = M v made here (kept up to kKeepTrain bytes)
+  char* tr = nullptr;      // training: sources r = M v made here (kept as KeepTrain says)
   size_t tr_bytes = 0;
   char* tl = nullptr;      // training: the loss of every step
   size_t tl_bytes = 0;
@@ -577,7 +577,8 @@ struct dirac_ptc {
 namespace dirac {
 namespace {
 
-constexpr size_t kKeepTrain = (size_t)256 << 20;
+// what a network keeps of its training buffers between calls: sources, loss history
+constexpr size_t kKeepTrain = (size_t)256 << 20, kKeepLoss = (size_t)1 << 20;
 constexpr int DSC_PARTIAL = MAXB + 8;
 constexpr int NORM_BLOCKS = 152;
 constexpr size_t DSC_DOUBLES = DSC_PARTIAL + (size_t)MAXB * NORM_BLOCKS;
@@ -597,6 +598,24 @@ int grow(dirac_ptc* n, char** p, size_t* have, size_t need) {
   *have = need;
   return DIRAC_OK;
 }
+
+// On every way out of a training call: waits for the launches that use the kept buffers (the
+// next call may come on another stream) and gives back what is above the bounds.
+struct KeepTrain {
+  dirac_ptc* n;
+  cudaStream_t st;
+  static void trim(char*& p, size_t& have, size_t keep) {
+    if (have <= keep) return;
+    cudaFree(p);
+    p = nullptr;
+    have = 0;
+  }
+  ~KeepTrain() {
+    cudaStreamSynchronize(st);
+    trim(n->tr, n->tr_bytes, kKeepTrain);
+    trim(n->tl, n->tl_bytes, kKeepLoss);
+  }
+};
 
 int check_net(dirac_ptc* n) {
   dirac_ctx* c = n->c;
@@ -931,6 +950,7 @@ extern "C" int dirac_ptc_train(dirac_ptc* n, const void* const* r, const void* c
   dirac_ctx* c = n->c;
   cudaStream_t st = (cudaStream_t)stream;
   const int B = std::min(P->batch, npairs);
+  const KeepTrain keep{n, st};
   // r_i = M v_i (FP32) when the caller gives only v
   // (a cudaMalloc and a cudaFree of both buffers per call cost a tenth of a short training)
   std::vector<const char*> rs(npairs);
@@ -979,11 +999,6 @@ extern "C" int dirac_ptc_train(dirac_ptc* n, const void* const* r, const void* c
       cudaMemcpy(loss, dloss, P->steps * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
     rc = cuda_check(c, "PTC train");
   cudaStreamSynchronize(st);
-  if (n->tr_bytes > kKeepTrain) {
-    cudaFree(n->tr);
-    n->tr = nullptr;
-    n->tr_bytes = 0;
-  }
   if (rc == DIRAC_OK) rc = cuda_check(c, "PTC train");
   return rc;
 }
