@@ -17,7 +17,7 @@ namespace dirac {
 
 void launch_wilson_ds(const WilsonArg& a, cudaStream_t st) {
   constexpr int T = WilsonShape<P64DS>::threads;
-  const int n = 2 * a.g.Vh;
+  const int n = full_sites(a.g.Vh);
   wilson_kernel<P64DS, 18, true><<<(n + T - 1) / T, T, 0, st>>>(a);
 }
 
