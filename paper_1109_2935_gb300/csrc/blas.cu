@@ -644,10 +644,10 @@ __global__ void __launch_bounds__(kThreads, MinBlocks<Op>::value) blas_map_kerne
 }
 
 // Sums of three values over a block, left in sum[0..2] of shared memory (valid after the
-// call). Warp k < 3 adds value k: 7 + 5 dependent FP64 additions. FP64 instructions issue at
-// one per 64 cycles and scheduler on this part whatever the active lanes, so shuffles in
-// all 8 warps followed by a serial pass over their results (39 per warp and 24 in thread 0)
-// took 1.7 us of every block; this takes 0.4.
+// call). Warp k < 3 adds value k: 7 additions in a tree, then 5 over the lanes. FP64
+// instructions issue at one per 64 cycles and scheduler on this part whatever the active
+// lanes, so shuffles in all 8 warps followed by a serial pass over their results (15
+// additions per warp, then 24 in thread 0) took 1.7 us of every block; this takes 0.4.
 struct RedShared {
   double v[3][kThreads];
   double sum[3];
