@@ -183,8 +183,13 @@ __device__ __forceinline__ void stag_hop(const StagArg& a, const int x[4], int c
 // neighbouring lanes; the sum passes from lane to lane in the order of LANES = 1, so the
 // results are the same bits. A small lattice is bound by the latency of a thread's 16 hops
 // (2 to 3 of them in flight), which four lanes share.
+// Nine CTAs per SM of the one-lane FP32 / FP16 form (56 registers; 18 reals spill two to
+// four): the loads in flight are what the warps hold. Left to itself the compiler takes 64 to
+// 72. Two launches, us, unset -> 9: 48^3x96 12-real FP32 1616 -> 1568 (10 CTAs 1555 to 1559),
+// FP16 1009 -> 965 (10: 972); 24^4 18-real FP32 92 -> 63, FP16 47 -> 35 (10: 37).
+template <int PREC, int LANES> constexpr int kStagCtas = PREC != P64 && LANES == 1 ? 9 : 0;
 template <int PREC, int RL, int LANES>
-__global__ void __launch_bounds__(128) staggered_kernel(const StagArg a) {
+__global__ void __launch_bounds__(128, (kStagCtas<PREC, LANES>)) staggered_kernel(const StagArg a) {
   pdl_begin();
   using T = typename Real<PREC>::T;
   const Geom& g = a.g;
