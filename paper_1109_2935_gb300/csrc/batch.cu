@@ -1,10 +1,10 @@
 // Batched application of the Wilson-clover operator: many right-hand sides on one
 // lattice, and several lattices of different sizes, in one persistent launch.
 //
-// A CTA works on tiles of 32 sites x RG right-hand sides (blockDim = (32, RG)): warp y
-// applies M to right-hand side rg*RG + y on the tile's 32 sites, so the links and the
-// clover of those sites are fetched from DRAM once and served to the other RG-1 warps
-// from L1. Every output site runs the same stencil code as the single-RHS kernel, so
+// A CTA works on tiles of 32 sites x RG right-hand sides (blockDim = (32, RG / NR)): warp y
+// applies M to NR (1 or 2) right-hand sides from rg*RG + y*NR on the tile's 32 sites, so the
+// links and the clover of those sites are fetched from DRAM once and served to the other
+// warps from L1. Every output site runs the same stencil code as the single-RHS kernel, so
 // results are bitwise identical. The tile shape (RG and the number of resident CTAs)
 // is chosen per batch plan by timing the candidates once (the autotuner below), and a
 // plan can record its launches in a CUDA graph for replay. With FP16 storage the plan

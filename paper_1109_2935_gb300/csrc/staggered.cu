@@ -283,8 +283,9 @@ static void launch_stag_lanes(int recon, const StagArg& a, cudaStream_t st) {
 }
 
 // Up to this many output sites four lanes share a site. Measured (two launches, us, one lane
-// -> four): FP32 4,096 sites 16.6 -> 9.7, 13,824 16.6 -> 12.5, 32,768 16.6 -> 20.7; FP16
-// 13,824 16.6 -> 12.5, 32,768 16.6 -> 16.5; FP64 4,096 57.6 -> 24.8, 13,824 59.7 -> 61.6.
+// -> four): FP32 4,096 sites 10.4 -> 8.1, 13,824 11.2 -> 8.3, 16,384 10.6 -> 9.7, 32,768 12.2 ->
+// 18.3; FP16 13,824 11.7 -> 8.3, 32,768 12.6 -> 11.3; FP64 4,096 53 -> 21, 8,192 53 -> 39, 13,824
+// 54.4 -> 55.3.
 template <int PREC> constexpr int kStagSplitSites = PREC == P64 ? 8192 : 16384;
 
 template <int PREC>

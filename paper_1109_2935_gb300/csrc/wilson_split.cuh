@@ -151,11 +151,11 @@ __global__ void __launch_bounds__(32) wilson_split64_kernel(const WilsonArg a) {
     *reinterpret_cast<double2*>((par ? a.out[1] : a.out[0]) + ((size_t)k * Vh + cb) * 16) = make_double2(out.r, out.i);
 }
 
-// Up to this many output sites the split form runs. Measured (M / hop block, us, one thread
-// per site -> split): 256 sites 40.0 / 31.7 -> 7.2 / 6.2, 4,096 40.3 / 31.7 -> 19.5 / 16.2,
-// 8,192 40.4 / 31.9 -> 34.7 / 29, 20,736 77.3 / 60 -> 86.0 / 72: with the chip full, its 2 x
-// larger integer and shared-memory work and the 4 idle lanes of the second phase cost more
-// than the shorter chain saves.
+// Up to this many output sites the split form runs. Measured (us, one thread per site ->
+// split): M 256 sites 39.7 -> 7.0, 4,096 39.7 -> 18.8, 8,192 39.7 -> 34.1, 12,288 39.9 -> 53.3; hop
+// block 128 sites 31.0 -> 6.3, 4,096 31.0 -> 15.5, 8,192 31.0 -> 28.2, 10,368 31.2 -> 36.6: with the
+// chip full, its 2 x larger integer and shared-memory work and the 4 idle lanes of the second
+// phase cost more than the shorter chain saves.
 constexpr int kSplitSites = 8192;
 
 template <int R>
